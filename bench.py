@@ -51,7 +51,6 @@ NCU_TRAFFIC = {
     # one ncu --set full capture per kernel on gmm16-5m (9,999,947 triangles),
     # scaled x2.0000 by triangle count to a gmm16-10m launch
     "bytes": {"walk": int((311.370 + 70.850) * 1e6 * 19999948 / 9999947),
-              "succ": int((232.247 + 105.619) * 1e6 * 19999948 / 9999947),
               "out_write": int((90.156 + 27.965) * 1e6 * 19999948 / 9999947),
               "label_class": int((130.077 + 80.119) * 1e6 * 19999948 / 9999947),
               "label_max": int((200.068 + 8.866) * 1e6 * 19999948 / 9999947),
@@ -120,13 +119,10 @@ def algorithmic_bytes(name: str, s: dict) -> float:
         "label_class": 12 * m + 2 * m + 12 * m,
         # label byte in, seed list and each seed's entry half-edge out
         "seed_write": m + 8 * ns,
-        # label bytes and every tf word once, the successor of every frontier
-        # half-edge out
-        "succ": m + 12 * m + 4 * nv0,
-        # per polygon its entry half-edge in and its output record (count, length,
-        # pos) out, per vertex succ + origin in and pool out, and start, length,
-        # tips and tip for each polygon with tips
-        "walk": 4 * ns + 12 * nv0 + 16 * ns + 16 * s.get("ntp", 0),
+        # every tf word once; per polygon its terminal half-edge in and its output
+        # record (count, length, pos) out, per vertex its origin in and pool out, and
+        # start, length, tips and tip for each polygon with tips
+        "walk": 12 * m + 4 * ns + 8 * nv0 + 16 * ns + 16 * s.get("ntp", 0),
         # per polygon its piece count and length
         "out_tiles": 8 * ns,
         # per polygon record in, pool in, offsets and vertices out
@@ -353,7 +349,7 @@ def run_ours(args, dist: Dist) -> dict | None:
     # algorithmic bytes and against the survey's estimate of the traversal phase's
     # bytes (about 35 B per triangle: twin, label and origin reads over the visited
     # half-edges, the vertex and offset writes)
-    trav = [k for k in ("succ", "walk") if k in kernels]
+    trav = [k for k in ("walk",) if k in kernels]
     tr_ms = sum(kernels[k]["ms"] for k in trav)
     tr_bytes = sum(kernels[k]["alg_bytes"] for k in trav)
     tr_survey = 35 * m

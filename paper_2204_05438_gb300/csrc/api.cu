@@ -51,12 +51,11 @@ struct polylla_mesh {
 
   uint8_t* lab = nullptr;
   int* seeds = nullptr;
-  int* entry = nullptr;   // per seed: entry half-edge of its region (or -1 - t)
+  int* entry = nullptr;   // per seed: terminal half-edge, where its walk enters
   int* lepp_region = nullptr;  // per triangle: seed of its longest-edge path's end
   int* lepp_depth = nullptr;   // per triangle: links of that path
   int* trivertex = nullptr;    // per vertex: smallest half-edge leaving it, or -1
   bool trivertex_valid = false;
-  int* succ = nullptr;    // per frontier half-edge: boundary successor | tip flag
   int* tf = nullptr;      // twin | frontier bit, per half-edge (written by the label phase)
   int* loc = nullptr;     // per half-edge: member index inside a long-polygon block
   int* vstamp = nullptr;  // per vertex: "endpoint of a split edge" stamp
@@ -179,7 +178,7 @@ struct Range {
 };
 
 void free_all(polylla_mesh* h) {
-  void* ptrs[] = {h->lab,      h->seeds,     h->succ,      h->tf,
+  void* ptrs[] = {h->lab,      h->seeds,     h->tf,
                   h->loc,      h->vstamp,    h->Lg.poly,   h->P.start,    h->P.len,
                   h->P.ntip,   h->P.pcnt,    h->P.pbase,    h->P.flen,
                   h->P.pos,    h->F.pos,     h->F.len,     h->F.h,        h->pool.v,
@@ -240,7 +239,6 @@ polylla_status alloc_derived(polylla_mesh* h) {
   if (e == cudaSuccess) e = dalloc(&(ptr), (cnt))
   ALLOC(h->lab, m + 4);
   ALLOC(h->seeds, m);
-  ALLOC(h->succ, 3 * m);
   ALLOC(h->entry, m);
   ALLOC(h->lepp_region, m);
   ALLOC(h->lepp_depth, m);
@@ -299,7 +297,6 @@ long long derived_bytes(long long n, long long m) {
   bytes += ((long long)sizeof(*(ptr)) * ((cnt) < 1 ? 1 : (long long)(cnt)) + 511) / 512 * 512
   COUNT(c.lab, m + 4);
   COUNT(c.seeds, m);
-  COUNT(c.succ, 3 * m);
   COUNT(c.entry, m);
   COUNT(c.tf, 3 * m);
   COUNT(c.loc, 3 * m);
@@ -395,26 +392,18 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
   // counters of this pass start at zero: right after the seeds they are (the label
   // phase cleared them); after a traversal pass they are cleared here
   // the kernel chain continues without a gap where the previous operation on the
-  // stream is its predecessor kernel: succ right after the seeds, the walk right
-  // after succ (not in timing mode, where events sit between the kernels)
+  // stream is its predecessor kernel: the walk right after the seeds (not in timing
+  // mode, where events sit between the kernels)
   const bool pdl = !h->timing && h->phase == kSeeded;
-  const bool succ_runs = repair == 0 || h->phase < kTraversed;
   if (h->phase != kSeeded) {
     const size_t first = offsetof(Counters, n_vtx_trav);
     const size_t last = offsetof(Counters, seed_ticket);
     POLY_TRY(cuda_status(cudaMemsetAsync(reinterpret_cast<char*>(h->C) + first, 0, last - first, s)));
   }
-  if (succ_runs) {
-    const int gt = grid_for(h, M.m, kBlock);
-    POLY_TRY(launch(h, "succ", s, [&] {
-      return launch_succ(M, h->lab, h->tf, h->succ, h->C, gt, s, pdl);
-    }));
-  }
-  const int gw = grid_for(h, M.m, 4 * 256);
+  const int gw = grid_for(h, M.m, kWalkThreads / 2);
   POLY_TRY(launch(h, "walk", s, [&] {
-    return launch_walk(M, h->tf, h->entry, h->succ, h->P, h->pool, h->Lg, h->Dl, h->Dm,
-                       h->walk_cap, repair, M.m < kSmallMeshTri ? 3 : 0, h->C, gw, s,
-                       !h->timing && succ_runs);
+    return launch_walk(M, h->tf, h->entry, h->P, h->pool, h->Lg, h->Dl, h->Dm, h->walk_cap,
+                       repair, M.m < kSmallMeshTri ? 3 : 0, h->C, gw, s, pdl);
   }));
   // repair_one (this stream), repair_multi and long (side streams) at once
   const bool fork = !h->timing && h->overlap;
@@ -427,18 +416,18 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
     s2 = h->side[1];
   }
   POLY_TRY(launch(h, "long", s1, [&] {
-    return launch_long(M, h->lab, h->tf, h->seeds, h->succ, h->P, h->F, h->pool, h->Lg, h->Lg2,
+    return launch_long(M, h->lab, h->tf, h->seeds, h->P, h->F, h->pool, h->Lg, h->Lg2,
                        h->loc, h->vstamp, 2 * h->epoch + repair, repair, h->long_mode, h->C,
                        h->sms, s1);
   }));
   if (repair) {
     POLY_TRY(launch(h, "repair_multi", s2, [&] {
-      return launch_repair_multi(M, h->lab, h->tf, h->succ, h->P, h->F, h->pool, h->Dm,
+      return launch_repair_multi(M, h->lab, h->tf, h->P, h->F, h->pool, h->Dm,
                                  h->rare_paths, h->C,
                                  h->sms, s2);
     }));
     POLY_TRY(launch(h, "repair_one", s, [&] {
-      return launch_repair_one(M, h->lab, h->tf, h->succ, h->P, h->F, h->pool, h->Dl,
+      return launch_repair_one(M, h->lab, h->tf, h->P, h->F, h->pool, h->Dl,
                                h->rare_paths, h->C, h->sms, s, !h->timing);
     }));
   }
@@ -452,8 +441,8 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
   // starts at zero with the pass's counters)
   const int gt = grid_for(h, M.m, kPolyTile);
   return launch(h, "out_write", s, [&] {
-    return launch_final_write(h->P, h->F, h->pool, h->out_status, off, vtx, h->obase, M.m, h->C,
-                              gt, s);
+    return launch_final_write(M, h->tf, h->P, h->F, h->pool, h->out_status, off, vtx, h->obase,
+                              h->C, gt, s);
   });
 }
 

@@ -5,7 +5,7 @@
 // pieces.  One single-pass scan over the polygons' (piece count, vertex count)
 // replaces the paper's AtomicAdd on i_Gmesh / i_Gpos, and each polygon's pieces
 // are copied to their offsets in the same pass.
-#include "polylla_internal.cuh"
+#include "walk.cuh"
 
 namespace polylla {
 
@@ -31,14 +31,28 @@ __device__ __forceinline__ void out_counts(const PolyArrays& P, long long i, lon
 // end marker.  The status words clean themselves: the block that completes the
 // last look-back (C->out_done counts them) clears them and the count.
 constexpr int kSub = 4;
+
+// Every frontier half-edge's turn ends, checked by the whole grid (a corrupt mesh
+// only: out of line, so that the copy kernel does not pay registers for it).
+__device__ __noinline__ void check_turns(const int* tf, int H, Counters* C) {
+  for (long long h = blockIdx.x * (long long)blockDim.x + threadIdx.x; h < H;
+       h += (long long)gridDim.x * blockDim.x) {
+    if (tf[h] >= 0) continue;
+    long long steps = 0;
+    if (turn_tf(tf, (int)h, H, steps, H) < 0) set_error(C, POLYLLA_ERR_LIMIT, 50);
+  }
+}
+
 constexpr int kOutTile = kSub * kPolyTile;
 
-__global__ void __launch_bounds__(kBlock, 5) k_final_write(PolyArrays P, FinalPieces F, Pool pool,
+__global__ void __launch_bounds__(kBlock, 5) k_final_write(DevMesh M, const int* tf, PolyArrays P,
+                                                        FinalPieces F, Pool pool,
                                                         unsigned long long* status,
                                                         long long* __restrict__ off,
                                                         int* __restrict__ vtx,
-                                                        long long* __restrict__ obase, long long m,
+                                                        long long* __restrict__ obase,
                                                         Counters* C) {
+  const long long m = M.m;
   __shared__ long long s_src[kSub][kBlock];  // pool position of each polygon (or -1)
   __shared__ int s_len[kSub][kBlock], s_pc[kSub][kBlock];
   __shared__ long long s_xc[kSub][kBlock], s_xl[kSub][kBlock];  // in-warp exclusive sums
@@ -46,6 +60,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_final_write(PolyArrays P, FinalPi
   __shared__ long long s_tile, s_p, s_v;
   __shared__ int s_clear;
   const long long n = C->n_seeds;
+  if (C->n_vtx_trav != C->n_front) check_turns(tf, (int)(3 * m), C);
   const long long ntiles = (n + kOutTile - 1) / kOutTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (;;) {
@@ -191,13 +206,13 @@ __global__ void __launch_bounds__(kBlock, 5) k_final_write(PolyArrays P, FinalPi
   }
 }
 
-cudaError_t launch_final_write(const PolyArrays& P, const FinalPieces& F, const Pool& pool,
-                               unsigned long long* status, long long* off, int* vtx,
-                               long long* obase, long long m, Counters* C, int grid,
+cudaError_t launch_final_write(const DevMesh& M, const int* tf, const PolyArrays& P,
+                               const FinalPieces& F, const Pool& pool, unsigned long long* status,
+                               long long* off, int* vtx, long long* obase, Counters* C, int grid,
                                cudaStream_t s) {
   static std::atomic<int> cap{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_final_write), kBlock, 0, grid, &cap);
-  k_final_write<<<grid, kBlock, 0, s>>>(P, F, pool, status, off, vtx, obase, m, C);
+  k_final_write<<<grid, kBlock, 0, s>>>(M, tf, P, F, pool, status, off, vtx, obase, C);
   return cudaGetLastError();
 }
 

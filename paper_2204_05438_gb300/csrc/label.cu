@@ -254,9 +254,9 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // them) clears them and the count, so nothing has to be zeroed before the next
 // run; the ticket counter C->seed_ticket starts at zero with the label phase's
 // counters.
-// With `entry` non-null, also the entry half-edge of each seed's region for the
-// walk: 3t + k for the first frontier edge k of t (label bits 2-4), or -1 - t when
-// t has no frontier edge (the walk then turns around t's first vertex).
+// With `entry` non-null, also the terminal half-edge 3t + k of each seed t (label
+// bits 0-1), where the walk enters its region.  The frontier half-edges (label bits
+// 2-4) are counted in C->n_front.
 constexpr int kSeedPer = 16;
 constexpr int kSeedSpan = kBlock * kSeedPer;   // triangles per sub-tile
 constexpr int kSeedSub = 4;                    // sub-tiles per look-back tile
@@ -321,6 +321,14 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
       if (lane == 31) sw[j][warp] = x;
     }
     __syncthreads();
+    unsigned nf = 0;
+#pragma unroll
+    for (int j = 0; j < kSeedSub; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) nf += __popc(w[j][q] & 0x1c1c1c1cu);
+    nf = __reduce_add_sync(0xffffffffu, nf);
+    if (lane == 0 && nf)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_front), (unsigned long long)nf);
     int sub_total[kSeedSub];
     int total = 0;
 #pragma unroll
@@ -356,10 +364,9 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
         const int i = __ffs(sm) - 1;
         sm &= sm - 1;
         const unsigned wq = i < 8 ? (i < 4 ? w[j][0] : w[j][1]) : (i < 12 ? w[j][2] : w[j][3]);
-        const unsigned fr = (wq >> (8 * (i & 3) + 2)) & 7u;
         const int t = (int)(t0 + i);
         s_seed[pos] = t;
-        s_entry[pos] = fr ? 3 * t + (__ffs(fr) - 1) : -1 - t;
+        s_entry[pos] = 3 * t + (int)((wq >> (8 * (i & 3))) & 3u);
         ++pos;
       }
       __syncthreads();

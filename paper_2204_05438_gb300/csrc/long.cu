@@ -11,8 +11,8 @@
 //      neither of its triangles), so the search goes down it
 //      from the seed without a visited set and ends after (longest-edge
 //      propagation depth + 1) levels;
-//   2. maps each half-edge's successor to a member index, finds the canonical
-//      start by a block reduction;
+//   2. finds each half-edge's successor by turning and maps it to a member index,
+//      finds the canonical start by a block reduction;
 //   3. without reparation (or tips): ranks the cycle from its start by pointer
 //      jumping in shared memory (log2(length) rounds) and writes the members in
 //      cycle order to the pool;
@@ -231,8 +231,7 @@ __device__ void long_fallback(const DevMesh& M, uint8_t* lab, int* tf, int t0, l
 // for this block size goes (with the counter n_over) instead of the sequential path.
 template <int THREADS, int LM, int LT>
 __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, int* tf,
-                                                  const int* __restrict__ seeds,
-                                                  const int* __restrict__ succ, PolyArrays P,
+                                                  const int* __restrict__ seeds, PolyArrays P,
                                                   FinalPieces F, Pool pool, LongList Lg,
                                                   const long long* n_list, LongList over,
                                                   long long* n_over, int* __restrict__ loc,
@@ -351,15 +350,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
     int ib = -1;
     for (int a = threadIdx.x; a < L; a += blockDim.x) {
       const int h = mem[a];
-      const int sg = succ[h];
-      const int g = sg & kSuccMask;
-      int b = ((unsigned)g < (unsigned)H) ? loc[g] : -1;
+      long long steps = 0;
+      const int g = turn_tf(tf, h, H, steps, limit);
+      int b = g >= 0 ? loc[g] : -1;
       if (b < 0 || b >= L || mem[b] != g) {
         s_fail = 1;
         b = a;
       }
       R0[a] = b;
-      if (sg & kTipFlag) tip_bar[atomicAdd(&s_nt, 1)] = h;
+      if (g >= 0 && g == tf_twin(tf[h])) tip_bar[atomicAdd(&s_nt, 1)] = h;
       const unsigned long long key = he_key(M.tri, h);
       if (key < kb) {
         kb = key;
@@ -487,8 +486,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
     const int ns = s_ns;
     const int N = L + 2 * ns;
     if (s_fail || N > kLM) {
-      // no split edge has been marked yet: the large blocks, or the sequential path
+      // no split edge has been marked yet: the large blocks, or the sequential path,
+      // which count the polygon themselves
       if (threadIdx.x == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_vtx_trav), 0ull - (unsigned long long)L);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tips), 0ull - (unsigned long long)nt);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tip_polys), ~0ull);
         if (over.poly && !s_fail) {
           const long long q =
               (long long)atomicAdd(reinterpret_cast<unsigned long long*>(n_over), 1ull);
@@ -524,17 +527,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
     unsigned long long* kb2 = reinterpret_cast<unsigned long long*>(R4); // R4..R5
     for (int a = threadIdx.x; a < N; a += blockDim.x) {
       const int h = mem[a];
-      int g;
-      if (vstamp[M.tri[he_next(h)]] == vst) {
+      int b;
+      if (a >= L || vstamp[M.tri[he_next(h)]] == vst) {
         long long steps = 0;
-        g = turn_tf(tf, h, H, steps, limit);
+        const int g = turn_tf(tf, h, H, steps, limit);
+        b = g >= 0 ? loc[g] : -1;
+        if (b < 0 || b >= N || mem[b] != g) {
+          s_fail = 1;
+          b = a;
+        }
       } else {
-        g = succ[h] & kSuccMask;
-      }
-      int b = ((unsigned)g < (unsigned)H) ? loc[g] : -1;
-      if (b < 0 || b >= N || mem[b] != g) {
-        s_fail = 1;
-        b = a;
+        b = R0[a];  // its turn as before the splits
       }
       na[a] = b;
       R6[a] = b;
@@ -728,8 +731,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
 
 template <int THREADS, int LM, int LT>
 cudaError_t launch_long_t(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
-                          const int* succ, const PolyArrays& P, const FinalPieces& F,
-                          const Pool& pool, const LongList& Lg, const long long* n_list,
+                          const PolyArrays& P, const FinalPieces& F, const Pool& pool,
+                          const LongList& Lg, const long long* n_list,
                           const LongList& over, long long* n_over, int* loc, int* vstamp,
                           int epoch, int repair, Counters* C, int grid, cudaStream_t s) {
   const size_t smem = sizeof(int) * (size_t)long_smem_ints<LM, LT>();
@@ -740,32 +743,32 @@ cudaError_t launch_long_t(const DevMesh& M, uint8_t* lab, int* tf, const int* se
   static std::atomic<int> cap{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_long<THREADS, LM, LT>), THREADS, smem,
                        grid, &cap);
-  k_long<THREADS, LM, LT><<<grid, THREADS, smem, s>>>(M, lab, tf, seeds, succ, P, F, pool, Lg,
+  k_long<THREADS, LM, LT><<<grid, THREADS, smem, s>>>(M, lab, tf, seeds, P, F, pool, Lg,
                                                       n_list, over, n_over, loc, vstamp, epoch,
                                                       repair, C);
   return cudaGetLastError();
 }
 
-cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds, const int* succ,
+cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
                         const PolyArrays& P, const FinalPieces& F, const Pool& pool,
                         const LongList& Lg, const LongList& Lg2, int* loc, int* vstamp, int epoch,
                         int repair, int mode, Counters* C, int sms, cudaStream_t s) {
   const LongList none{nullptr, 0};
   if (mode == 0)  // large blocks only
-    return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, succ, P, F, pool, Lg,
+    return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, P, F, pool, Lg,
                                                  &C->n_long, none, nullptr, loc, vstamp, epoch,
                                                  repair, C, sms, s);
   // small blocks (mode 1) or one warp per polygon (mode 2) first; the regions
   // they cannot hold, in large blocks
   cudaError_t e =
-      mode == 2 ? launch_long_t<32, kWarpLM, kWarpLT>(M, lab, tf, seeds, succ, P, F, pool, Lg,
+      mode == 2 ? launch_long_t<32, kWarpLM, kWarpLT>(M, lab, tf, seeds, P, F, pool, Lg,
                                                       &C->n_long, Lg2, &C->n_long2, loc, vstamp,
                                                       epoch, repair, C, 32 * sms, s)
                 : launch_long_t<kSmallThreads, kSmallLM, kSmallLT>(
-                      M, lab, tf, seeds, succ, P, F, pool, Lg, &C->n_long, Lg2, &C->n_long2, loc,
+                      M, lab, tf, seeds, P, F, pool, Lg, &C->n_long, Lg2, &C->n_long2, loc,
                       vstamp, epoch, repair, C, 16 * sms, s);
   if (e != cudaSuccess) return e;
-  return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, succ, P, F, pool, Lg2,
+  return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, P, F, pool, Lg2,
                                                &C->n_long2, none, nullptr, loc, vstamp, epoch,
                                                repair, C, sms, s);
 }

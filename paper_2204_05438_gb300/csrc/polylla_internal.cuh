@@ -31,6 +31,7 @@ constexpr int kScanThreads = 1024;
 // Device-resident counters of one pipeline run (zeroed by the label phase).
 struct Counters {
   long long n_seeds;
+  long long n_front;      // frontier half-edges of the labelled mesh
   long long n_vtx_trav;   // total length of the traversal polygons
   long long n_tip_polys;  // polygons with >= 1 barrier-edge tip
   long long n_tips;
@@ -172,7 +173,7 @@ __device__ __forceinline__ T block_sum(T v, T* sh) {
 }
 
 // ---------------------------------------------- programmatic dependent launch
-// The kernels of the chain label_max -> label_class -> seed_write -> succ -> walk
+// The kernels of the chain label_max -> label_class -> seed_write -> walk
 // run back to back on one stream.  A chain kernel may be launched with
 // programmatic stream serialization (launch_chain, pdl = true) when the previous
 // operation on the stream is a kernel: its launch is then processed while the
@@ -252,7 +253,8 @@ cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, Counters* C, int gr
 // the stream is a kernel)
 cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters* C, int grid,
                                cudaStream_t s, bool pdl);
-// The ascending seed list (and entries, if non-null) and C->n_seeds in one pass:
+// The ascending seed list (and each seed's terminal half-edge, if entry is
+// non-null), C->n_seeds and C->n_front in one pass:
 // look-back over `status` (seed_tiles(m) words, zero at the first use; left zero)
 // with tickets from C->seed_ticket (zero at the start).
 cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
@@ -304,33 +306,28 @@ struct LongList {
   long long cap;
 };
 
-// lab: the label bytes (their frontier bits select the half-edges to turn)
-cudaError_t launch_succ(const DevMesh& M, const uint8_t* lab, const int* tf, int* succ,
-                        Counters* C, int grid, cudaStream_t s, bool pdl);
 // One thread per seed: walk (<= kWalkCap) and, if `repair`, list polygons with
 // tips.  cap: polygons longer than cap (16, 32, 48 or 64) go to the long-polygon
 // blocks; with tips_to_long > 0 (small meshes), so do polygons with that many tips
 // or more when `repair` (the block splits their tips in parallel; one thread would
 // split them one after another).
 constexpr long long kSmallMeshTri = 1ll << 16;  // meshes below this: tips_to_long = 3
-cudaError_t launch_walk(const DevMesh& M, int* tf, const int* entry, const int* succ,
-                        const PolyArrays& P, const Pool& pool, const LongList& Lg,
-                        const LongList& D1, const LongList& Dm, int cap, int repair,
-                        int tips_to_long, Counters* C, int grid, cudaStream_t s, bool pdl);
+cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,
+                        const Pool& pool, const LongList& Lg, const LongList& D1,
+                        const LongList& Dm, int cap, int repair, int tips_to_long, Counters* C,
+                        int grid, cudaStream_t s, bool pdl);
 // One thread per polygon with one tip / with several tips (listed by k_walk).
-cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const int* succ,
-                              const PolyArrays& P, const FinalPieces& F, const Pool& pool,
-                              const LongList& D1, int rare, Counters* C, int sms,
-                              cudaStream_t s, bool pdl);
-cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const int* succ,
-                                const PolyArrays& P, const FinalPieces& F, const Pool& pool,
-                                const LongList& Dm, int rare, Counters* C, int sms,
-                                cudaStream_t s);
+cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
+                              const FinalPieces& F, const Pool& pool, const LongList& D1, int rare,
+                              Counters* C, int sms, cudaStream_t s, bool pdl);
+cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
+                                const FinalPieces& F, const Pool& pool, const LongList& Dm,
+                                int rare, Counters* C, int sms, cudaStream_t s);
 // One block per long polygon: gather, rank and, if `repair`, split.  mode 0:
 // large blocks only; mode 1: small blocks first, the regions they cannot hold
 // (listed in Lg2) then in large blocks; mode 2: the same with one-warp blocks
 // first.
-cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds, const int* succ,
+cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
                         const PolyArrays& P, const FinalPieces& F, const Pool& pool,
                         const LongList& Lg, const LongList& Lg2, int* loc, int* vstamp, int epoch,
                         int repair, int mode, Counters* C, int sms, cudaStream_t s);
@@ -338,9 +335,12 @@ cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seed
 // 1024-polygon tile, zero at the first use and left zero) and the copy; also
 // C->n_poly, C->n_vtx and off[n_poly].
 // obase (nullable): per traversal polygon, the index of its first output polygon.
-cudaError_t launch_final_write(const PolyArrays& P, const FinalPieces& F, const Pool& pool,
-                               unsigned long long* status, long long* off, int* vtx,
-                               long long* obase, long long m, Counters* C, int grid,
+// A corrupt (unvalidated) mesh may have frontier half-edges that no seed's walk
+// meets; when the walks' vertices do not add up to the frontier half-edges, every
+// turn is checked to end (an endless one is POLYLLA_ERR_LIMIT).
+cudaError_t launch_final_write(const DevMesh& M, const int* tf, const PolyArrays& P,
+                               const FinalPieces& F, const Pool& pool, unsigned long long* status,
+                               long long* off, int* vtx, long long* obase, Counters* C, int grid,
                                cudaStream_t s);
 // The twin array from tri (scratch: cnt n, start n + 1, adj 3m pairs; the tile words).
 cudaError_t launch_build_twin(const int* tri, long long m, long long n, int* twin, int* cnt,

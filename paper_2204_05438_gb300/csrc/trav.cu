@@ -1,19 +1,15 @@
 // Traversal (Section 3.2.2, Algorithms 3 and 4) and, for ordinary polygons,
 // reparation (Section 3.2.3, Algorithm 5) in one pass.
 //
-//   k_succ  for each frontier half-edge, the next frontier half-edge of its
-//           region's boundary (PolyConstruction's turn), with the barrier-edge
-//           tip flag; each warp compacts the frontier half-edges of 256
-//           triangles and turns them one per lane.
-//   k_walk  one thread per seed: enter the region (at the entry half-edge the
-//           seed kernel found), chase succ around the cycle (at most kWalkCap
-//           vertices, staged in shared memory), note the canonical start and the
-//           tips.  A polygon without tips (or any, when no reparation is asked
-//           for) is copied, rotated to its canonical start, into the vertex pool,
-//           whose space is handed out per warp.  A polygon
-//           with tips is listed -- one tip (about 90% of them) or several -- so
-//           that the dependent loads of a split do not stall the 31 other lanes of
-//           its warp; a longer one is left to one thread block (long.cu).
+//   k_walk  a warp takes 32 seeds: the triangles of their regions, from each terminal
+//           edge down the region's longest-edge tree, then every boundary edge's
+//           place in its polygon (at most kWalkCap vertices) from the subtree sizes,
+//           the canonical starts and the tips.  A polygon without tips (or any, when
+//           no reparation is asked for) is copied, rotated to its canonical start,
+//           into the vertex pool, whose space is handed out per warp.  A polygon
+//           with tips is listed -- one tip (about 90% of them) or several -- so that
+//           the dependent loads of a split do not stall its warp; a longer one is
+//           left to one thread block (long.cu).
 //   k_repair_one    one thread per polygon with one tip: split it and cut the
 //           two pieces out of the vertex sequence the walk left in the pool.
 //   k_repair_multi  one thread per polygon with several tips: the cycle becomes
@@ -24,122 +20,9 @@
 // (final.cu); the pool order does not matter.
 #include "walk.cuh"
 
+#include <cstddef>
+
 namespace polylla {
-
-// Each warp takes a chunk of 32 * PER consecutive triangles at a time (PER = 8
-// on large meshes): their frontier half-edges (label bits 2-4, PER triangles per
-// lane) are compacted into the warp's list in shared memory by a warp scan, in
-// increasing order, and then turned 32 at a time, one per lane: no lane idles on a
-// half-edge that is not frontier, and the 32 turns of a round start at
-// neighbouring half-edges.  On a mesh with fewer 256-triangle chunks than the
-// grid has warps, smaller chunks (PER = 4, 2, 1) give every warp work, so a warp
-// turns fewer rounds one after another.
-template <int PER>
-__device__ __forceinline__ unsigned long long load_lab(const uint8_t* __restrict__ lab,
-                                                       long long t0, long long m) {
-  unsigned long long v = 0;
-  if (t0 + PER <= m && (reinterpret_cast<uintptr_t>(lab + t0) & (PER - 1)) == 0) {
-    if (PER == 8) {
-      const uint2 w = __ldg(reinterpret_cast<const uint2*>(lab + t0));
-      v = (unsigned long long)w.x | ((unsigned long long)w.y << 32);
-    } else if (PER == 4) {
-      v = __ldg(reinterpret_cast<const unsigned*>(lab + t0));
-    } else if (PER == 2) {
-      v = __ldg(reinterpret_cast<const unsigned short*>(lab + t0));
-    } else {
-      v = __ldg(lab + t0);
-    }
-  } else {
-    for (int i = 0; i < PER && t0 + i < m; ++i)
-      v |= (unsigned long long)__ldg(lab + t0 + i) << (8 * i);
-  }
-  return v;
-}
-
-template <int PER>
-__global__ void __launch_bounds__(kBlock) k_succ(DevMesh M, const uint8_t* __restrict__ lab,
-                                                 const int* __restrict__ tf,
-                                                 int* __restrict__ succ, Counters* C) {
-  constexpr int kChunk = 32 * PER;
-  // half-edge offsets inside the chunk (< 3 * kChunk): 16 bits leave the L1 the
-  // turns read from
-  __shared__ unsigned short s_list[kBlock / 32][3 * kChunk];
-  pdl_wait();  // the label bytes and tf words
-  pdl_launch_dependents();
-  const long long m = M.m;
-  const int H = (int)(3 * m);
-  const int lane = threadIdx.x & 31;
-  unsigned short* list = s_list[threadIdx.x >> 5];
-  const long long nchunks = (m + kChunk - 1) / kChunk;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  // the label bytes of this lane's PER triangles of chunk ch (loaded one chunk ahead)
-  auto load = [&](long long ch) -> unsigned long long {
-    if (ch >= nchunks) return 0;
-    return load_lab<PER>(lab, ch * kChunk + (long long)lane * PER, m);
-  };
-  long long ch = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  unsigned long long next = load(ch);
-  for (; ch < nchunks; ch += nwarps) {
-    const unsigned long long bytes = next;
-    next = load(ch + nwarps);
-    // bit 3i + k: half-edge k of the lane's triangle i is frontier
-    unsigned mask = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) mask |= (unsigned)((bytes >> (8 * i + 2)) & 7u) << (3 * i);
-    const int c = __popc(mask);
-    int incl = c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    int pos = incl - c;
-    const int o0 = 3 * PER * lane;  // this lane's first half-edge in the chunk
-    while (mask) {
-      const int s = __ffs(mask) - 1;
-      mask &= mask - 1;
-      list[pos++] = (unsigned short)(o0 + s);
-    }
-    __syncwarp();
-    const int hc = (int)(3 * ch * kChunk);  // the chunk's first half-edge
-    for (int j = lane; j < total; j += 32) {
-      const int h = hc + list[j];
-      const int x = __ldg(tf + h);
-      int cur = he_next(h);
-      int y = __ldg(tf + cur);
-      for (int steps = 0; y >= 0;) {
-        if (y >= H || ++steps > H) {
-          set_error(C, POLYLLA_ERR_LIMIT, 50);
-          cur = h;
-          break;
-        }
-        cur = he_next(y);
-        y = __ldg(tf + cur);
-      }
-      succ[h] = (cur == tf_twin(x)) ? (cur | kTipFlag) : cur;
-    }
-    __syncwarp();
-  }
-}
-
-template <int PER>
-cudaError_t launch_succ_t(const DevMesh& M, const uint8_t* lab, const int* tf, int* succ,
-                          Counters* C, int grid, cudaStream_t s, bool pdl) {
-  static std::atomic<int> cap{0};
-  grid = resident_grid(reinterpret_cast<const void*>(k_succ<PER>), kBlock, 0, grid, &cap);
-  return launch_chain(k_succ<PER>, grid, kBlock, 0, s, pdl, M, lab, tf, succ, C);
-}
-
-cudaError_t launch_succ(const DevMesh& M, const uint8_t* lab, const int* tf, int* succ,
-                        Counters* C, int grid, cudaStream_t s, bool pdl) {
-  // the largest chunk that still gives every warp of the grid at least one
-  const long long warps = (long long)grid * (kBlock / 32);
-  if (M.m >= 256 * warps) return launch_succ_t<8>(M, lab, tf, succ, C, grid, s, pdl);
-  if (M.m >= 128 * warps) return launch_succ_t<4>(M, lab, tf, succ, C, grid, s, pdl);
-  if (M.m >= 64 * warps) return launch_succ_t<2>(M, lab, tf, succ, C, grid, s, pdl);
-  return launch_succ_t<1>(M, lab, tf, succ, C, grid, s, pdl);
-}
 
 // Warp-aggregated allocation: each lane asks for `need` entries; one atomic per
 // warp.  All 32 lanes must call it.
@@ -165,191 +48,446 @@ __device__ __forceinline__ long long warp_alloc(long long* counter, int need) {
 // several-tip kernel's node list.
 constexpr int kRsMaxSplit = 8;
 
-// Warp-aggregated list append: each lane with `want` gets its own slot of the
-// list counted by `counter` (one atomic per warp, slots in lane order), the
-// others -1.  All 32 lanes must call it.
-__device__ __forceinline__ long long warp_append(long long* counter, bool want) {
-  const unsigned b = __ballot_sync(0xffffffffu, want);
-  if (b == 0) return -1;
+// The walk of 32 seeds by a warp.  The non-frontier edges of a region form its
+// longest-edge tree (every triangle but the terminal pair hangs from the neighbour
+// across its longest edge), so the boundary cycle is the tree's tour: the subtree of
+// the seed's triangle, entered through its terminal edge e0, then the one across e0
+// (only e0 itself when e0 is a border edge).  A triangle entered through half-edge e
+// contributes the boundary across n1 = next(e), then across n2 = prev(e): the edge
+// itself if it is frontier, else the subtree behind it.  The warp does not follow the
+// tour; it places every boundary edge by the sizes of the subtrees before it:
+//
+//   1. the triangles of the 32 regions go through one queue in shared memory, 32 a
+//      pass, one lane each: two independent loads (tf[n1], tf[n2]), the children
+//      appended (their queue indices in link[]);
+//   2. the passes backwards: each triangle's boundary edges, from its children's;
+//   3. the passes forwards: each triangle's place in its polygon, its children's, and
+//      its frontier edges into he[], polygon after polygon;
+//   4. the origins gathered, a lane per boundary edge; a lane per polygon scans them
+//      for the smallest (origin, half-edge) and the tips; then every lane stores its
+//      edges' origins, each polygon turned to start there, in one stretch of the pool.
+//
+// What bounds it: the latency of the queue's passes, ten on average for the 212
+// triangles of 32 regions, and the instructions issued (3,000 a warp and 32 seeds, 60
+// % of the issue slots); DRAM is at a quarter.  One lane per polygon that follows
+// precomputed successors runs as long as the longest of its warp's 32 polygons (21
+// steps where the mean is 8.6) with scattered loads at every step, and the successors
+// took a pass of their own.  gmm16-10m (20M triangles): 0.369 ms, against 0.188 ms for
+// the successors and 0.338 ms for that walk; 1M uniform points 0.062 against 0.087 ms;
+// the same with shuffled triangles 0.072 against 0.103; 200,000 mixture points 0.029
+// against 0.038.  A lane (or two) per polygon on the tour itself took 0.58-0.65 ms.
+// A warp whose regions do not fit the queue (0.3 %) leaves out those already too long
+// for a walk, or takes half as many seeds at a time.
+constexpr int kWalkWarps = kWalkThreads / 32;
+constexpr int kWalkQ = 288;              // triangles of a warp's regions
+constexpr int kWalkE = kWalkQ + 2 * 32;  // a region of T triangles has T + 2 boundary edges
+constexpr int kWalkPasses = 64;          // one region of at most kWalkCap - 2 triangles fits
+constexpr int kWalkLeast = 16;           // seeds a warp on a small mesh
+constexpr int kGather = 5;               // loads in flight a lane in step 4
+constexpr int kTipSlots = 48;            // tips of a warp's polygons (two on average)
+constexpr unsigned kKidA = 0x400, kKidB = 0x800;  // link: children, below them (10 bits)
+constexpr int kCorner = 12;  // the first child's queue index, above them the entry's corner
+static_assert(kWalkQ + 64 < (int)kKidA && kWalkQ >= kWalkCap && 2 * kWalkQ >= kWalkE &&
+                  kWalkPasses >= kWalkCap,
+              "links hold queue indices, any one region fits, the vertices fit v");
+
+struct WalkBuf {
+  int he[kWalkE];  // boundary half-edges, polygon after polygon
+  union {
+    struct {
+      int e[kWalkQ];                // the queue: entry half-edge of each triangle,
+      unsigned short link[kWalkQ];  // its children and its corner,
+      unsigned short cp[kWalkQ];    // its subtree's boundary edges, then its place
+    } q;
+    int v[kWalkE];  // step 4: origins of he
+  } u;
+  unsigned short p0[kWalkPasses];  // first queue index of each pass
+  int tip_h[kTipSlots];  // tips (candidates, then -1 if none): half-edge,
+  int tip_at[kTipSlots]; // polygon << 16 | place in the polygon
+  // per polygon that is not empty, in lane order: its tips, its place (and length << 10),
+  // its smallest vertex, where that is, its lane
+  int nt[32], info[32], least[32], rank[32];
+  unsigned char lane[32];
+  unsigned starts[kWalkE / 32 + kGather];  // bit j: a polygon starts at place j
+  int one[64], multi[64];        // polygons with one tip, with several, to be listed
+  int tn;
+};
+
+// The warp's n buffered polygons appended to a list, one atomic for all; returns 0.
+__device__ __forceinline__ int list_flush(const int* buf, int n, const LongList& D,
+                                          long long* counter, Counters* C) {
   const int lane = threadIdx.x & 31;
-  const int leader = __ffs(b) - 1;
-  unsigned long long base = 0;
-  if (lane == leader)
-    base = atomicAdd(reinterpret_cast<unsigned long long*>(counter), (unsigned long long)__popc(b));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  return want ? (long long)base + __popc(b & ((1u << lane) - 1u)) : -1;
+  __syncwarp();
+  unsigned long long at = 0;
+  if (lane == 0)
+    at = atomicAdd(reinterpret_cast<unsigned long long*>(counter), (unsigned long long)n);
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if ((long long)at + n > D.cap) set_error(C, POLYLLA_ERR_LIMIT, 55);
+  for (int k = lane; k < n; k += 32)
+    if ((long long)at + k < D.cap) D.poly[at + k] = buf[k];
+  __syncwarp();
+  return 0;
 }
 
-// Triangle of a seed's entry word (3t + k, or -1 - t)
-__device__ __forceinline__ long long entry_tri(int e) { return e >= 0 ? e / 3 : -1 - (long long)e; }
-
-// L2 prefetch of the whole 128-byte lines inside [p, p + bytes) (the partial
-// lines at either end are left out, so no address outside the range is touched),
-// spread over the block
-__device__ __forceinline__ void prefetch_l2(const void* p, long long bytes) {
-  const uintptr_t lo = (reinterpret_cast<uintptr_t>(p) + 127) & ~(uintptr_t)127;
-  const uintptr_t hi = (reinterpret_cast<uintptr_t>(p) + (uintptr_t)bytes) & ~(uintptr_t)127;
-  for (uintptr_t c = lo + 128 * (uintptr_t)threadIdx.x; c < hi; c += 128 * (uintptr_t)blockDim.x)
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(c));
-}
-
-
-__global__ void __launch_bounds__(kWalkThreads) k_walk(DevMesh M, int* tf,
-                                                       const int* __restrict__ entry,
-                                                       const int* __restrict__ succ, PolyArrays P,
-                                                       Pool pool, LongList Lg, LongList D1,
-                                                       LongList Dm, int cap, int repair,
-                                                       int tips_to_long, Counters* C) {
-  // staging transposed (word q of thread x at q * blockDim + x): the lanes of a
-  // warp, writing the same position in lockstep, hit 32 different banks
-  extern __shared__ int sbuf[];
-  pdl_wait();  // the successors, seeds and entries
-  int* my = sbuf + threadIdx.x;
-  const long long n = C->n_seeds;
+__global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* __restrict__ tf,
+                                                          const int* __restrict__ entry,
+                                                          PolyArrays P, Pool pool, LongList Lg,
+                                                          LongList D1, LongList Dm, int cap,
+                                                          int repair, int tips_to_long,
+                                                          Counters* C) {
+  extern __shared__ __align__(16) unsigned char walk_smem[];
+  pdl_wait();  // the tf words, seeds and entries
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+  WalkBuf& B = reinterpret_cast<WalkBuf*>(walk_smem)[warp];
+  const int* __restrict__ tri = M.tri;
+  const int n = (int)C->n_seeds;  // below 2^29
   const int H = (int)(3 * M.m);
-  const long long limit = 3 * M.m + 3;
+  // polygons with 2 to this many tips get tip records
+  const int most_rec = tips_to_long > 0 ? min(tips_to_long - 1, kRsMaxSplit) : kRsMaxSplit;
   unsigned st_len = 0, st_tips = 0, st_tippolys = 0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += stride) {
-    const long long i = base + threadIdx.x;
-    // the next iteration's seeds lie in one run of triangles (seeds ascend): the
-    // successor words of that run go to L2 now, while this iteration walks (the
-    // same for tri, or with a margin around the run, was slower)
-    if (base + stride < n) {
-      const long long nb = base + stride;
-      const long long ne = (nb + blockDim.x < n ? nb + blockDim.x : n) - 1;
-      const long long t0 = entry_tri(__ldg(entry + nb));
-      long long t1 = entry_tri(__ldg(entry + ne));
-      t1 = t1 >= M.m ? M.m - 1 : t1;
-      if (t1 >= t0) {
-        prefetch_l2(succ + 3 * t0, 12 * (t1 - t0 + 1));
+  // 32 seeds a warp and round, or fewer while that leaves no warp without any: on a
+  // small mesh a warp's chain of passes is the kernel's time (200,000 mixture points, 60,204
+  // seeds: 28.7 us against 39 with 32 seeds a warp)
+  const int warps = (int)gridDim.x * kWalkWarps;
+  int per = 32;
+  while (per > kWalkLeast && n <= (per >> 1) * warps) per >>= 1;
+  int width = per;  // seeds taken at a time
+  int n1 = 0, nm = 0;  // entries of the warp's list buffers
+  for (int base = ((int)blockIdx.x * kWalkWarps + warp) * per; base < n; base += warps * per) {
+    const int i = base + lane;
+    const int e0 = lane < per && i < n ? __ldg(entry + i) : -1;
+    int x0 = e0 >= 0 ? __ldg(tf + e0) : -1;
+    bool big = false;  // too long for a walk: left to a thread block
+    for (int b0 = 0; b0 < per && base + b0 < n;) {
+      const bool taken = e0 >= 0 && lane >= b0 && lane < b0 + width;
+      if (taken && x0 >= H) {
+        set_error(C, POLYLLA_ERR_LIMIT, 52);
+        x0 = -1;
       }
-    }
-    int len = 0, ntips = 0, tip_h = -1, tip_s = 0, rank0 = 0, start = 0;
-    bool closed = false, is_long = false;
-    if (i < n) {
-      int e = entry[i];
-      if (e < 0) e = region_entry_tf(tf, -1 - e, H, limit);
-      if (e < 0) {
-        set_error(C, POLYLLA_ERR_LIMIT, 51);
-      } else {
-        unsigned long long best = ~0ull;
-        int tipv = 0x7fffffff;
-        int h = e;
-        bool ok = true;
-        do {
-          const int o = M.tri[h];
-          my[len * kWalkThreads] = o;
-          const unsigned long long key = ((unsigned long long)(unsigned)o << 32) | (unsigned)h;
-          if (key < best) {
-            best = key;
-            rank0 = len;
+      const bool mine = taken && !big;
+      const bool inner = mine && x0 >= 0;  // the terminal edge has a far side
+      const unsigned ma = __ballot_sync(full, mine), mb = __ballot_sync(full, inner);
+      const int ra = __popc(ma & lt), rb = __popc(ma) + __popc(mb & lt);  // the roots
+      int hi = __popc(ma) + __popc(mb);
+      if (mine) B.u.q.e[ra] = e0;
+      if (inner) B.u.q.e[rb] = x0;
+      B.nt[lane] = 0;
+      if (lane < kWalkE / 32 + kGather) B.starts[lane] = 0;
+      if (lane == 0) B.tn = 0;
+      __syncwarp();
+      // ---- 1. the queue
+      int np = 0, lo = 0;
+      bool overflow = false;
+      while (lo < hi) {
+        if (lane == 0) B.p0[np] = (unsigned short)lo;
+        const int x = lo + lane;
+        int a = -1, b = -1, k = 0;
+        if (x < hi) {
+          const int e = B.u.q.e[x];
+          k = (int)((unsigned)e % 3u);
+          a = __ldg(tf + (k == 2 ? e - 2 : e + 1));
+          b = __ldg(tf + (k == 0 ? e + 2 : e - 1));
+          if (max(a, b) >= H) {
+            set_error(C, POLYLLA_ERR_LIMIT, 52);
+            a = b = -1;
           }
-          const int sg = succ[h];
-          const int g = sg & kSuccMask;
-          if (sg & kTipFlag) {
-            ++ntips;
-            // tip record k (its half-edge and step), staged from the top while
-            // the origins below have not reached it
-            if (ntips <= kRsMaxSplit && cap - 2 * ntips > len) {
-              my[(cap - 2 * ntips) * kWalkThreads] = h;
-              my[(cap - 2 * ntips + 1) * kWalkThreads] = len;
-            }
-            const int b = M.tri[g];  // dest(h) = origin(twin(h))
-            if (b < tipv) {
-              tipv = b;
-              tip_h = h;
-              tip_s = len;
-            }
-          }
-          ++len;
-          if ((unsigned)g >= (unsigned)H) {
-            ok = false;
-            break;
-          }
-          h = g;
-        } while (h != e && len < cap);
-        closed = ok && h == e;
-        is_long = ok && !closed;
-        // several tips on a small mesh: the block kernel splits them in parallel
-        if (closed && repair && tips_to_long > 0 && ntips >= tips_to_long) {
-          closed = false;
-          is_long = true;
         }
-        if (!ok) set_error(C, POLYLLA_ERR_LIMIT, 52);
-        start = (int)(best & 0xffffffffu);
+        const unsigned da = __ballot_sync(full, a >= 0), db = __ballot_sync(full, b >= 0);
+        const int ca = hi + __popc(da & lt) + __popc(db & lt);  // the first child
+        const int cb = ca + (a >= 0);
+        const int end = hi + __popc(da) + __popc(db);
+        if (end > kWalkQ || np == kWalkPasses - 1) {
+          overflow = true;
+          break;
+        }
+        if (x < hi)
+          B.u.q.link[x] = (unsigned short)(ca | (a >= 0 ? kKidA : 0) | (b >= 0 ? kKidB : 0) |
+                                           k << kCorner);
+        if (a >= 0) B.u.q.e[ca] = a;
+        if (b >= 0) B.u.q.e[cb] = b;
+        __syncwarp();
+        lo = min(lo + 32, hi);
+        hi = end;
+        ++np;
       }
-    }
-    const bool split = closed && repair && ntips > 0;
-    // a one-tip polygon's vertex sequence goes to the pool too: its split cuts
-    // the two pieces out of it
-    const bool seq = split && ntips == 1;
-    // a polygon with 2..kRsMaxSplit tips whose records all stayed above its
-    // origins: the sequence and the records (rotated tip index, tip half-edge)
-    // go to the pool, where the several-tip kernel also writes its pieces
-    const bool rec = split && ntips >= 2 && ntips <= kRsMaxSplit && len + 2 * ntips <= cap;
-    const int need = (closed && (!split || seq)) ? len : (rec ? len + 2 * ntips : 0);
-    const long long off = warp_alloc(&C->pool_alloc, need);
-    // list slots, one atomic per warp and list
-    const long long jl = warp_append(&C->n_long, i < n && is_long);
-    const long long j1 = warp_append(&C->n_defer, i < n && split && ntips == 1);
-    const long long jm = warp_append(&C->n_multi, i < n && split && ntips > 1);
-    if (i >= n) continue;
-    if (is_long) {
-      P.pcnt[i] = 0;
-      P.flen[i] = 0;
-      if (jl < Lg.cap) Lg.poly[jl] = (int)i;
-      continue;
-    }
-    // start, length and tips are read only by the reparation kernels
-    P.pcnt[i] = 0;
-    P.flen[i] = 0;
-    if (!closed) continue;
-    st_len += len;
-    st_tips += ntips;
-    st_tippolys += ntips > 0;
-    if (need) {  // the sequence, rotated to the canonical start
-      if (off + need > pool.cap) {
-        set_error(C, POLYLLA_ERR_LIMIT, 53);
-        // its list slot is taken: a record the split kernels skip
-        if (seq && j1 < D1.cap) {
-          P.len[i] = 0;
-          D1.poly[j1] = (int)i;
+      if (overflow) {  // the triangles not followed count as leaves
+        for (int x = lo + lane; x < hi; x += 32) B.u.q.cp[x] = 2;
+        __syncwarp();
+      }
+      // ---- 2. boundary edges of every subtree
+      for (int p = np - 1, end = overflow ? lo : hi; p >= 0; --p) {
+        const int first = B.p0[p];
+        const int x = first + lane;
+        if (x < end) {
+          const unsigned l = B.u.q.link[x];
+          const unsigned ca = l & (kKidA - 1), cb = ca + (l & kKidA ? 1 : 0);
+          int c = 2;
+          if (l & kKidA) c += B.u.q.cp[ca] - 1;
+          if (l & kKidB) c += B.u.q.cp[cb] - 1;
+          B.u.q.cp[x] = (unsigned short)c;
         }
-        if (rec && jm < Dm.cap) {
-          P.len[i] = 0;
-          Dm.poly[jm] = (int)i;
+        end = first;
+        __syncwarp();
+      }
+      // ---- the polygons' lengths and places
+      const int na = mine ? B.u.q.cp[ra] : 0;
+      int L = mine ? na + (inner ? B.u.q.cp[rb] : 1) : 0;
+      const bool over = L > cap;
+      big |= over;
+      if (overflow) {
+        if (!__any_sync(full, over)) {
+          if (width == 1) big |= taken;  // (a single region that fits never gets here)
+          else width >>= 1;
         }
+        __syncwarp();
         continue;
       }
-      int* out = pool.v + off;
-      int r = rank0;
-      for (int q = 0; q < len; ++q) {
-        out[q] = my[r * kWalkThreads];
-        if (++r == len) r = 0;
+      if (over) L = 0;
+      int first = L;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(full, first, d);
+        if (lane >= d) first += y;
       }
-      for (int k = 1; rec && k <= ntips; ++k) {
-        const int st = my[(cap - 2 * k + 1) * kWalkThreads];
-        out[len + 2 * (k - 1)] = st >= rank0 ? st - rank0 : st - rank0 + len;
-        out[len + 2 * (k - 1) + 1] = my[(cap - 2 * k) * kWalkThreads];
+      const int E = __shfl_sync(full, first, 31);
+      first -= L;
+      long long off = 0;
+      if (lane == 0 && E > 0)
+        off = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->pool_alloc),
+                                   (unsigned long long)E);
+      if (mine) {
+        B.u.q.cp[ra] = over ? 0xffff : (unsigned short)first;
+        if (inner) B.u.q.cp[rb] = over ? 0xffff : (unsigned short)(first + na);
+        else if (!over) B.he[first + na] = e0;
       }
-      P.pos[i] = off;
+      __syncwarp();
+      // ---- 3. the boundary edges in order
+      for (int p = 0; p < np; ++p) {
+        const int x = B.p0[p] + lane;
+        if (x < (p + 1 < np ? (int)B.p0[p + 1] : hi)) {
+          const unsigned l = B.u.q.link[x];
+          const unsigned ca = l & (kKidA - 1), cb = ca + (l & kKidA ? 1 : 0), k = l >> kCorner;
+          const int at = B.u.q.cp[x];
+          const int e = B.u.q.e[x];
+          int bt = at;
+          if (at != 0xffff) {
+            if (l & kKidA) bt += B.u.q.cp[ca];
+            else B.he[bt++] = k == 2 ? e - 2 : e + 1;
+            if (!(l & kKidB)) B.he[bt] = k == 0 ? e + 2 : e - 1;
+          }
+          if (l & kKidA) B.u.q.cp[ca] = (unsigned short)at;
+          if (l & kKidB) B.u.q.cp[cb] = (unsigned short)bt;
+        }
+        __syncwarp();
+      }
+      // ---- 4. the vertices.  The polygon of place j is the number of polygons that
+      //         start at or before it (starts: a bit per place)
+      const unsigned some = __ballot_sync(full, L > 0);
+      const int ord = __popc(some & lt);
+      if (L) {
+        B.info[ord] = first | L << 10;
+        B.least[ord] = 0x7fffffff;
+        B.rank[ord] = 0;
+        atomicOr(&B.starts[first >> 5], 1u << (first & 31));
+      }
+      __syncwarp();
+      const unsigned upto = lt << 1 | 1u;
+      for (int j0 = 0, poly = -1; j0 < E; j0 += 32 * kGather) {
+        int o[kGather];
+#pragma unroll
+        for (int w = 0; w < kGather; ++w) {
+          const int j = j0 + 32 * w + lane;
+          if (j < E) o[w] = __ldg(tri + B.he[j]);
+        }
+#pragma unroll
+        for (int w = 0; w < kGather; ++w) {
+          const int j = j0 + 32 * w + lane;
+          const unsigned starts = B.starts[(j0 >> 5) + w];
+          if (j < E) {
+            B.u.v[j] = o[w];
+            atomicMin(&B.least[poly + __popc(starts & upto)], o[w]);
+          }
+          poly += __popc(starts);
+        }
+      }
+      __syncwarp();
+      // where each polygon's smallest vertex is (count << 16 | place in the polygon),
+      // and where a vertex repeats two steps on: a tip a, b, a if its half-edge a->b is
+      // followed by its twin
+#pragma unroll 1
+      for (int j0 = 0, poly = -1; j0 < E; j0 += 32) {
+        const unsigned starts = B.starts[j0 >> 5];
+        const int j = j0 + lane;
+        if (j < E) {
+          const int s = poly + __popc(starts & upto);
+          const int inf = B.info[s];
+          const int p0 = inf & 1023, l = inf >> 10;
+          const int v = B.u.v[j];
+          int j2 = j + 2;
+          if (j2 >= p0 + l) j2 -= l;
+          if (v == B.least[s]) atomicAdd(&B.rank[s], 0x10000 + j - p0);
+          if (v == B.u.v[j2]) {
+            const int k = atomicAdd(&B.tn, 1);
+            if (k < kTipSlots) B.tip_at[k] = s << 16 | (j - p0);
+          }
+        }
+        poly += __popc(starts);
+      }
+      __syncwarp();
+      int rank = L ? B.rank[ord] : 0;
+      if (rank >> 16 > 1) {  // it repeats: the smallest half-edge
+        const int least = B.least[ord];
+        int h = 0x7fffffff;
+        for (int q = 0; q < L; ++q)
+          if (B.u.v[first + q] == least && B.he[first + q] < h) {
+            h = B.he[first + q];
+            rank = q;
+          }
+      }
+      rank &= 0xffff;
+      const int tn = B.tn;
+      const int start = L ? B.he[first + rank] : 0;
+      for (int t0 = 0; t0 < min(tn, kTipSlots); t0 += 32) {
+        const int t = t0 + lane;
+        const bool live = t < min(tn, kTipSlots);
+        if (live) {
+          const int at = B.tip_at[t], inf = B.info[at >> 16];
+          const int q = at & 0xffff, p0 = inf & 1023, l = inf >> 10;
+          const int h = B.he[p0 + q];
+          const bool tip = tf_twin(__ldg(tf + h)) == B.he[p0 + (q + 1 < l ? q + 1 : 0)];
+          B.tip_h[t] = tip ? h : -1;
+          if (tip) atomicAdd(&B.nt[at >> 16], 1);
+        }
+      }
+      __syncwarp();
+      // the lists of polygons to split, kept in the warp's buffers until one is half full
+      const int ntips = L ? B.nt[ord] : 0;
+      // several tips on a small mesh: the block kernel splits them in parallel; it
+      // also takes the polygons of a warp whose tip list is full
+      const bool many =
+          L && (tn > kTipSlots || (repair && tips_to_long > 0 && ntips >= tips_to_long));
+      const bool is_long = taken && (big || many);
+      const bool split = repair && ntips > 0 && !many;
+      const bool rec = split && ntips >= 2 && ntips <= most_rec;
+      const unsigned m1 = __ballot_sync(full, split && ntips == 1);
+      const unsigned mm = __ballot_sync(full, split && ntips > 1);
+      if (split) {
+        if (ntips == 1) B.one[n1 + __popc(m1 & lt)] = i;
+        else B.multi[nm + __popc(mm & lt)] = i;
+      }
+      n1 += __popc(m1);
+      nm += __popc(mm);
+      // to the pool, each polygon turned to its canonical start: the polygon of an
+      // edge is the number of polygons that start at or before it
+      if (L) {
+        B.rank[ord] = rank;
+        B.lane[ord] = (unsigned char)lane;
+      }
+      __syncwarp();
+      off = __shfl_sync(full, off, 0);
+      const bool fits = off + E <= pool.cap;
+      if (!fits && lane == 0) set_error(C, POLYLLA_ERR_LIMIT, 53);
+      if (fits) {
+        int* out = pool.v + off;
+#pragma unroll 1
+        for (int j0 = 0, poly = -1; j0 < E; j0 += 32) {
+          const unsigned starts = B.starts[j0 >> 5];
+          const int j = j0 + lane;
+          if (j < E) {
+            const int s = poly + __popc(starts & upto);
+            const int inf = B.info[s];
+            int at = j - B.rank[s];
+            if (at < (inf & 1023)) at += inf >> 10;
+            out[at] = B.u.v[j];
+          }
+          poly += __popc(starts);
+        }
+      }
+      // ---- records and lists
+      long long roff = off + first;
+      if (__any_sync(full, rec)) {
+        // several tips: the sequence and the records (rotated tip index, tip
+        // half-edge) get space of their own, which the pieces overwrite
+        const long long o = warp_alloc(&C->pool_alloc, rec ? L + 2 * ntips : 0);
+        if (rec) roff = o;
+      }
+      // an entry of a list whose sequence is not in the pool is one of length 0,
+      // which the split kernels skip
+      const bool kept = fits && (!rec || roff + L + 2 * ntips <= pool.cap);
+      if (rec && !kept) set_error(C, POLYLLA_ERR_LIMIT, 53);
+      for (unsigned left = __ballot_sync(full, rec && kept); left; left &= left - 1) {
+        const int s = __ffs(left) - 1;
+        const int p0 = __shfl_sync(full, first, s), l = __shfl_sync(full, L, s);
+        const int pr = __shfl_sync(full, rank, s);
+        const long long po = __shfl_sync(full, roff, s);
+        for (int q = lane; q < l; q += 32)
+          pool.v[po + (q >= pr ? q - pr : q - pr + l)] = B.u.v[p0 + q];
+      }
+      if (repair) {
+        for (int t0 = 0; t0 < min(tn, kTipSlots); t0 += 32) {
+          const int t = t0 + lane;
+          const bool live = t < min(tn, kTipSlots) && B.tip_h[t] >= 0;
+          const int at = live ? B.tip_at[t] : 0;
+          const int s = at >> 16, owner = live ? B.lane[s] : 0;
+          const long long po = __shfl_sync(full, roff, owner);
+          const int how = __shfl_sync(full, (int)(split && kept) | (int)rec << 1, owner);
+          if (live && (how & 1)) {
+            const int inf = B.info[s], pr = B.rank[s];
+            const int p0 = inf & 1023, l = inf >> 10;
+            const int q = at & 0xffff;
+            const int b = B.u.v[p0 + (q + 1 < l ? q + 1 : 0)];  // the tip vertex
+            int order = 0;
+            bool lowest = true;
+            const bool one = B.nt[s] == 1;
+            for (int k = 0; k < min(tn, kTipSlots) && !one; ++k) {
+              if (B.tip_at[k] >> 16 != s || B.tip_h[k] < 0) continue;
+              const int qk = B.tip_at[k] & 0xffff;
+              order += k < t;
+              lowest &= B.u.v[p0 + (qk + 1 < l ? qk + 1 : 0)] >= b;
+            }
+            const int rot = q >= pr ? q - pr : q - pr + l;
+            const int ip = base + owner;
+            if (how & 2) {
+              pool.v[po + l + 2 * order] = rot;
+              pool.v[po + l + 2 * order + 1] = B.tip_h[t];
+            }
+            if (lowest) {
+              P.tip_h[ip] = B.tip_h[t];
+              if (one) P.pbase[ip] = rot;  // the tip's index in the sequence
+            }
+          }
+        }
+      }
+      if (taken) {
+        P.pcnt[i] = 0;
+        P.flen[i] = split || is_long || !fits ? 0 : L;
+        if (is_long) {
+          const long long d =
+              (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_long), 1ull);
+          if (d < Lg.cap) Lg.poly[d] = i;
+        } else {
+          P.pos[i] = roff;
+          st_len += L;
+          st_tips += ntips;
+          st_tippolys += ntips > 0;
+        }
+        if (split) {
+          P.start[i] = start;
+          P.len[i] = kept ? L : 0;
+          P.ntip[i] = ntips;
+          if (ntips > 1) P.pbase[i] = rec ? 1 : 0;  // several tips: records at pos, or none
+        }
+      }
+      __syncwarp();
+      if (n1 > 32) n1 = list_flush(B.one, n1, D1, &C->n_defer, C);
+      if (nm > 32) nm = list_flush(B.multi, nm, Dm, &C->n_multi, C);
+      b0 += width;
     }
-    if (split) {
-      P.start[i] = start;
-      P.len[i] = len;
-      P.ntip[i] = ntips;
-      P.tip_h[i] = tip_h;
-      if (seq) P.pbase[i] = tip_s >= rank0 ? tip_s - rank0 : tip_s - rank0 + len;
-      else P.pbase[i] = rec ? 1 : 0;  // several tips: records at pos, or none
-      LongList& D = (ntips == 1) ? D1 : Dm;
-      const long long d = (ntips == 1) ? j1 : jm;
-      if (d < D.cap) D.poly[d] = (int)i;
-      else set_error(C, POLYLLA_ERR_LIMIT, 55);
-      continue;
-    }
-    P.flen[i] = len;
+    width = min(per, 2 * width);
   }
+  if (n1) list_flush(B.one, n1, D1, &C->n_defer, C);
+  if (nm) list_flush(B.multi, nm, Dm, &C->n_multi, C);
   st_len = __reduce_add_sync(0xffffffffu, st_len);
   st_tips = __reduce_add_sync(0xffffffffu, st_tips);
   st_tippolys = __reduce_add_sync(0xffffffffu, st_tippolys);
@@ -361,21 +499,19 @@ __global__ void __launch_bounds__(kWalkThreads) k_walk(DevMesh M, int* tf,
   }
 }
 
-cudaError_t launch_walk(const DevMesh& M, int* tf, const int* entry, const int* succ,
-                        const PolyArrays& P, const Pool& pool, const LongList& Lg,
-                        const LongList& D1, const LongList& Dm, int cap, int repair,
-                        int tips_to_long, Counters* C, int grid, cudaStream_t s, bool pdl) {
+cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,
+                        const Pool& pool, const LongList& Lg, const LongList& D1,
+                        const LongList& Dm, int cap, int repair, int tips_to_long, Counters* C,
+                        int grid, cudaStream_t s, bool pdl) {
   if (cap < 16 || cap > kWalkCap || cap % 16) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(int) * (size_t)kWalkThreads * cap;
+  constexpr size_t smem = sizeof(WalkBuf) * kWalkWarps;
   static std::atomic<bool> attr[kMaxDevices];
-  const cudaError_t e = smem_limit_once(reinterpret_cast<const void*>(k_walk),
-                                        (int)(sizeof(int) * kWalkThreads * kWalkCap), attr);
+  const cudaError_t e = smem_limit_once(reinterpret_cast<const void*>(k_walk), (int)smem, attr);
   if (e != cudaSuccess) return e;
-  static std::atomic<int> resident[kWalkCap / 16 + 1] = {};
-  grid = resident_grid(reinterpret_cast<const void*>(k_walk), kWalkThreads, smem, grid,
-                       &resident[cap / 16]);
-  return launch_chain(k_walk, grid, kWalkThreads, smem, s, pdl, M, tf, entry, succ, P, pool, Lg, D1,
-                      Dm, cap, repair, tips_to_long, C);
+  static std::atomic<int> resident{0};
+  grid = resident_grid(reinterpret_cast<const void*>(k_walk), kWalkThreads, smem, grid, &resident);
+  return launch_chain(k_walk, grid, kWalkThreads, smem, s, pdl, M, tf, entry, P, pool, Lg, D1, Dm,
+                      cap, repair, tips_to_long, C);
 }
 
 __device__ __forceinline__ unsigned long long vkey(int origin, int h) {
@@ -386,7 +522,7 @@ constexpr int kSeqChunk = 4;  // sequence entries loaded at a time by the split 
 
 // One tip p = a->b, split along oj = b->x (tw = x->b), with q = turn(oj) and
 // pn = twin(p) = b->a.  The two pieces are
-//     oj, q, succ(q), ..., p          and          tw, pn, succ(pn), ..., pred(q)
+//     oj, q, turn(q), ..., p          and          tw, pn, turn(pn), ..., pred(q)
 // (the boundary walk with oj, tw frontier); the other frontier half-edges keep
 // their turns.  The walk left the polygon's vertex sequence v (from its canonical
 // start) in the pool and the tip's index t in it (v[t] = a, v[t+1] = b).  When x
@@ -395,13 +531,12 @@ constexpr int kSeqChunk = 4;  // sequence entries loaded at a time by the split 
 // (indices cyclic); each is written from its smallest vertex when that vertex
 // occurs once in it (then it is the canonical start).  Otherwise (x, or a piece's
 // smallest vertex, repeated: the canonical start needs half-edge ids) the two arcs
-// of the cycle are chased along succ at once, staged over v (arc 1 from the
-// front, arc 2 from the back), and each piece is copied from its canonical start.
+// of the cycle are walked by turning, staged over v (arc 1 from the front, arc 2
+// from the back), and each piece is copied from its canonical start.
 // Pool space: L + 2 for the pieces.
 __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, int* tf,
-                                                       const int* __restrict__ succ, PolyArrays P,
-                                                       FinalPieces F, Pool pool, LongList D1,
-                                                       int rare, Counters* C) {
+                                                       PolyArrays P, FinalPieces F, Pool pool,
+                                                       LongList D1, int rare, Counters* C) {
   pdl_wait();  // the walk's lists, records and sequences
   const long long nd = min(C->n_defer, D1.cap);
   const int H = (int)(3 * M.m);
@@ -538,11 +673,8 @@ __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, 
       bool a1 = true, a2 = true;
       unsigned long long b1 = vkey(b, oj), b2 = vkey(x, tw);
       for (int it = 0; (a1 || a2) && it < L; ++it) {
-        const int o1 = a1 ? M.tri[c1] : 0;
-        const int s1 = a1 ? succ[c1] : 0;
-        const int o2 = a2 ? M.tri[c2] : 0;
-        const int s2 = a2 ? succ[c2] : 0;
         if (a1) {
+          const int o1 = M.tri[c1];
           stage[n1] = o1;
           const unsigned long long k = vkey(o1, c1);
           ++n1;
@@ -551,9 +683,10 @@ __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, 
             r1 = n1;
           }
           if (c1 == tp) a1 = false;
-          else c1 = s1 & kSuccMask;
+          else c1 = turn_tf(tf, c1, H, steps, limit);
         }
         if (a2) {
+          const int o2 = M.tri[c2];
           ++n2;
           stage[L - n2] = o2;
           const unsigned long long k = vkey(o2, c2);
@@ -561,10 +694,10 @@ __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, 
             b2 = k;
             r2 = n2;
           }
-          c2 = s2 & kSuccMask;
-          if (c2 == g) a2 = false;
+          c2 = turn_tf(tf, c2, H, steps, limit);
+          if (c2 == tw) a2 = false;
         }
-        if ((unsigned)c1 >= (unsigned)H || (unsigned)c2 >= (unsigned)H) break;
+        if (c1 < 0 || c2 < 0) break;
       }
       if (a1 || a2 || n1 + n2 != L) {
         ++st_bad;
@@ -619,17 +752,16 @@ __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, 
 // none (x always has a frontier edge of the region besides the chord), so only
 // those two flags change.
 //
-// The node list comes from the walk's records when it left them (the origins
-// from the canonical start, and each tip's index and half-edge): the other
-// nodes' half-edges stay unknown (kSuccMask) unless needed.  q is the piece's
+// The node list comes from the walk's records (the origins from the canonical
+// start, and each tip's index and half-edge): the other nodes' half-edges stay
+// unknown (kSuccMask) unless needed.  q is the piece's
 // only node with origin x; when x occurs more than once in the piece, q is the
 // one whose successor's origin is dest(turn(oj)) (a directed edge occurs once in
 // a boundary).  A finished piece starts at its smallest vertex; when that vertex
 // occurs more than once, the piece's half-edges are found by turning from a node
 // whose half-edge is known (a chord), and the smallest (origin, half-edge) key
-// decides.  Without records the list is built by chasing the successors.  The
-// pieces are written over the records (as long as the polygon and its tip
-// records, at least its final length).
+// decides.  The pieces are written over the records (as long as the polygon and
+// its tip records, at least its final length).
 constexpr int kRsThreads = 64;
 constexpr int kRsNodes = kWalkCap + 2 * kRsMaxSplit;
 constexpr int kRsList = kRsMaxSplit + 2;
@@ -637,7 +769,6 @@ constexpr size_t kRsSmem =
     (size_t)kRsThreads * (kRsNodes * (2 * sizeof(int) + 2) + kRsList);
 
 __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t* lab, int* tf,
-                                                             const int* __restrict__ succ,
                                                              PolyArrays P, FinalPieces F,
                                                              Pool pool, LongList Dm, int rare,
                                                              Counters* C) {
@@ -682,7 +813,9 @@ __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t*
     } else {
       cnt = -1;
       bool bad = false;
-      if (rec) {  // the walk's records
+      if (!rec) {
+        bad = true;  // the walk leaves records for every such polygon
+      } else {
         const int* rv = pool.v + off;
         for (int j0 = 0; j0 < L; j0 += kSeqChunk) {
           int w[kSeqChunk];
@@ -706,21 +839,6 @@ __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t*
           }
           NH(ix) = hh | kTipFlag;
         }
-      } else {  // chase the successors from the canonical start
-        int h = P.start[i];
-        for (int j = 0; j < L; ++j) {
-          if ((unsigned)h >= (unsigned)H) {
-            bad = true;
-            break;
-          }
-          const int sg = succ[h];
-          NH(j) = h | (sg & kTipFlag);
-          NO(j) = M.tri[h];
-          NX(j) = (uint8_t)(j + 1 == L ? 0 : j + 1);
-          PV(j) = (uint8_t)(j == 0 ? L - 1 : j - 1);
-          h = sg & kSuccMask;
-        }
-        if (h != P.start[i]) bad = true;
       }
       int nn = kWalkCap;  // next chord node
       int count = 1;
@@ -896,19 +1014,18 @@ __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t*
     atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_turn), (unsigned long long)st_turn);
 }
 
-cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const int* succ,
-                              const PolyArrays& P, const FinalPieces& F, const Pool& pool,
+cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
+                              const FinalPieces& F, const Pool& pool,
                               const LongList& D1, int rare, Counters* C, int sms,
                               cudaStream_t s, bool pdl) {
   static std::atomic<int> cap{0};
   const int grid = resident_grid(reinterpret_cast<const void*>(k_repair_one), kBlock, 0,
                                  (long long)sms * 8, &cap);
-  return launch_chain(k_repair_one, grid, kBlock, 0, s, pdl, M, lab, tf, succ, P, F, pool, D1, rare,
-                      C);
+  return launch_chain(k_repair_one, grid, kBlock, 0, s, pdl, M, lab, tf, P, F, pool, D1, rare, C);
 }
 
-cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const int* succ,
-                                const PolyArrays& P, const FinalPieces& F, const Pool& pool,
+cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
+                                const FinalPieces& F, const Pool& pool,
                                 const LongList& Dm, int rare, Counters* C, int sms,
                                 cudaStream_t s) {
   static std::atomic<bool> attr[kMaxDevices];
@@ -917,7 +1034,7 @@ cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const i
   if (e != cudaSuccess) return e;
   const int per_sm = (int)((220 * 1024) / (kRsSmem + 1024));
   const int grid = sms * (per_sm < 1 ? 1 : per_sm);
-  k_repair_multi<<<grid, kRsThreads, kRsSmem, s>>>(M, lab, tf, succ, P, F, pool, Dm, rare, C);
+  k_repair_multi<<<grid, kRsThreads, kRsSmem, s>>>(M, lab, tf, P, F, pool, Dm, rare, C);
   return cudaGetLastError();
 }
 

@@ -10,11 +10,11 @@
 // contributes its origin vertex.  A turn reads one tf word per step: tf[g] < 0
 // iff g is frontier, and its low 31 bits are twin(g).
 //
-// The turn of every frontier half-edge is also precomputed into succ[h] (k_succ)
-// for the first walk; bit 31 of succ[h] flags a barrier-edge tip: succ(h) ==
-// twin(h), i.e. consecutive polygon vertices v_a, v_b, v_a with v_b = dest(h)
-// (Section 3.2.3).  Every loop is bounded and every index range-checked, so a
-// corrupt mesh ends in an error code, not a hang or a stray access.
+// A frontier half-edge h ends at a barrier-edge tip when its turn comes straight
+// back along its twin, i.e. consecutive polygon vertices v_a, v_b, v_a with
+// v_b = dest(h) (Section 3.2.3).  Every loop is bounded and every index
+// range-checked, so a corrupt mesh ends in an error code, not a hang or a stray
+// access.
 #pragma once
 
 #include "polylla_internal.cuh"
