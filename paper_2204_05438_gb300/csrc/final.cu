@@ -17,20 +17,31 @@ __device__ __forceinline__ void out_counts(const PolyArrays& P, long long i, lon
 }
 
 // Every polygon's output -- its pieces in order, for a split one -- lies in one
-// contiguous stretch of the pool, and the untouched polygons that one walk warp
-// pooled (32 consecutive seeds) lie back to back.  So a warp's 32 polygons form a
-// few runs that are contiguous both in the pool and in the output, broken where
-// a polygon was split or walked elsewhere; each run is copied by the whole warp,
-// coalesced.  Piece offsets are written by the polygon's own thread.
+// contiguous stretch of the pool, and the output of a warp's 32 polygons is one
+// contiguous stretch of the CSR.  The warp copies that stretch flat, a lane per vertex:
+// the vertex's polygon is the number of polygons that start at or before it (a bit per
+// polygon start in a 32-vertex window), and each polygon has one distance from its
+// place in the stretch to its place in the pool.  kOutLoads windows are loaded before
+// any is stored, so that a warp's ten windows take two round trips to L2, however its
+// polygons lie in the pool.
 //
-// A block takes kSub consecutive 256-polygon sub-tiles per ticket (one look-back
-// tile), so one block scan and one look-back serve 1024 polygons.  The tile
+// What bounds it: latency (a tile's records, its look-back, its copies).  Copying one
+// after another the runs that are contiguous in the pool as well took a round trip per
+// run, and the polygons that splits take out of the walk's order leave five or so of
+// them to a warp.  Times before and after, us: gmm16-10m 135 and 115, 1M uniform points
+// 35 and 28, 200,000 mixture points 29 and 14, 20,000 points with holes 22 and 11.
+//
+// A block takes SUB consecutive 256-polygon sub-tiles per ticket (one look-back tile):
+// four on large meshes, so that one look-back serves 1024 polygons (gmm16-10m 115 us
+// against 158 with one), one on small meshes, whose tiles would leave SMs idle (20,000
+// points: 11 us against 17; at 1M points, kOutSmall, 28 against 31).  The tile
 // offsets come from a look-back over `status` in the same pass (tiles in ticket
 // order; one word per tile packs the piece count << 33 | vertex count, exact
 // within the mesh size limits), and the last tile writes the totals and the CSR
 // end marker.  The status words clean themselves: the block that completes the
 // last look-back (C->out_done counts them) clears them and the count.
-constexpr int kSub = 4;
+constexpr int kOutLoads = 6;
+constexpr long long kOutSmall = 1ll << 21;  // triangles: 1,230 tiles of 256 polygons
 
 // Every frontier half-edge's turn ends, checked by the whole grid (a corrupt mesh
 // only: out of line, so that the copy kernel does not pay registers for it).
@@ -43,21 +54,25 @@ __device__ __noinline__ void check_turns(const int* tf, int H, Counters* C) {
   }
 }
 
-constexpr int kOutTile = kSub * kPolyTile;
 
-__global__ void __launch_bounds__(kBlock, 5) k_final_write(DevMesh M, const int* tf, PolyArrays P,
+template <int SUB>
+__global__ void __launch_bounds__(kBlock, SUB == 4 ? 6 : 5) k_final_write(DevMesh M, const int* tf, PolyArrays P,
                                                         FinalPieces F, Pool pool,
                                                         unsigned long long* status,
                                                         long long* __restrict__ off,
                                                         int* __restrict__ vtx,
                                                         long long* __restrict__ obase,
                                                         Counters* C) {
+  constexpr int kWarps = kBlock / 32;
+  constexpr long long kOutTile = SUB * kPolyTile;
+  constexpr long long kLen = (1ll << 33) - 1;  // counts << 33 | vertices
+  static_assert(SUB * kWarps <= 32, "one warp scans the warps' totals");
   const long long m = M.m;
-  __shared__ long long s_src[kSub][kBlock];  // pool position of each polygon (or -1)
-  __shared__ int s_len[kSub][kBlock], s_pc[kSub][kBlock];
-  __shared__ long long s_xc[kSub][kBlock], s_xl[kSub][kBlock];  // in-warp exclusive sums
-  __shared__ long long s_wc[kBlock / 32][kSub], s_wl[kBlock / 32][kSub];  // warp sums
-  __shared__ long long s_tile, s_p, s_v;
+  __shared__ long long s_src[SUB][kBlock], s_x[SUB][kBlock];  // pool place; in-warp sums
+  __shared__ int s_len[SUB][kBlock], s_pc[SUB][kBlock];
+  __shared__ long long s_sum[SUB * kWarps];  // per sub-tile and warp: total, then offsets
+  __shared__ long long s_dist[kWarps][32];
+  __shared__ long long s_tile;
   __shared__ int s_clear;
   const long long n = C->n_seeds;
   if (C->n_vtx_trav != C->n_front) check_turns(tf, (int)(3 * m), C);
@@ -70,59 +85,52 @@ __global__ void __launch_bounds__(kBlock, 5) k_final_write(DevMesh M, const int*
     const long long tile = s_tile;
     if (tile >= ntiles) break;
     // this thread's polygon in each sub-tile; every load issued before any use
-    int pcj[kSub], lj[kSub];
+    int pcj[SUB], lj[SUB];
 #pragma unroll
-    for (int j = 0; j < kSub; ++j) {
+    for (int j = 0; j < SUB; ++j) {
       const long long i = tile * kOutTile + (long long)j * kPolyTile + threadIdx.x;
       pcj[j] = i < n ? P.pcnt[i] : 0;
       lj[j] = i < n ? P.flen[i] : 0;
     }
 #pragma unroll
-    for (int j = 0; j < kSub; ++j) {
+    for (int j = 0; j < SUB; ++j) {
       const long long i = tile * kOutTile + (long long)j * kPolyTile + threadIdx.x;
       const long long src = i < n ? (pcj[j] == 0 ? P.pos[i] : F.pos[P.pbase[i]]) : -1;
       s_src[j][threadIdx.x] = src;
-      // the polygon's first vertex (and its line) to L2 while the tile waits for
-      // its look-back
-      if (src >= 0 && src < pool.cap) asm volatile("prefetch.global.L2 [%0];" ::"l"(pool.v + src));
       s_len[j][threadIdx.x] = lj[j];
       s_pc[j][threadIdx.x] = pcj[j];
-      long long xc = i < n ? (pcj[j] == 0 ? 1 : pcj[j]) : 0, xl = lj[j];
-      const long long c0 = xc, l0 = xl;
+      // the polygon's first vertex (and its line) to L2 while the tile waits for its
+      // look-back
+      if (src >= 0 && src < pool.cap) asm volatile("prefetch.global.L2 [%0];" ::"l"(pool.v + src));
+      const long long own = i < n ? (long long)max(pcj[j], 1) << 33 | lj[j] : 0;
+      long long x = own;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const long long yc = __shfl_up_sync(0xffffffffu, xc, d);
-        const long long yl = __shfl_up_sync(0xffffffffu, xl, d);
-        if (lane >= d) {
-          xc += yc;
-          xl += yl;
-        }
+        const long long y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
       }
-      s_xc[j][threadIdx.x] = xc - c0;
-      s_xl[j][threadIdx.x] = xl - l0;
-      if (lane == 31) {
-        s_wc[warp][j] = xc;
-        s_wl[warp][j] = xl;
-      }
+      s_x[j][threadIdx.x] = x - own;
+      if (lane == 31) s_sum[j * kWarps + warp] = x;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-      long long ac = 0, al = 0;
-      for (int j = 0; j < kSub; ++j)
-        for (int w = 0; w < kBlock / 32; ++w) {
-          ac += s_wc[w][j];
-          al += s_wl[w][j];
-        }
-      const long long ex = lookback_warp(status, tile, (ac << 33) | al, C);
-      if (threadIdx.x == 0) {
-        s_p = ex >> 33;
-        s_v = ex & ((1ll << 33) - 1);
+    if (warp == 0) {
+      const long long own = lane < SUB * kWarps ? s_sum[lane] : 0;
+      long long x = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+      }
+      const long long all = __shfl_sync(0xffffffffu, x, 31);
+      const long long ex = lookback_warp(status, tile, all, C);
+      if (lane < SUB * kWarps) s_sum[lane] = ex + x - own;
+      if (lane == 0) {
         // the last look-back to complete clears the status words for the next pass
         const unsigned long long done =
             atomicAdd(reinterpret_cast<unsigned long long*>(&C->out_done), 1ull);
         s_clear = done == (unsigned long long)(ntiles - 1);
         if (tile == ntiles - 1) {
-          const long long np = s_p + ac, nv = s_v + al;
+          const long long np = (ex + all) >> 33, nv = (ex + all) & kLen;
           C->n_poly = np;
           C->n_vtx = nv;
           if (np <= m) off[np] = nv;
@@ -131,72 +139,68 @@ __global__ void __launch_bounds__(kBlock, 5) k_final_write(DevMesh M, const int*
       }
     }
     __syncthreads();
-    long long bp = s_p, bv = s_v;  // offsets of sub-tile j's first polygon
-    for (int j = 0; j < kSub; ++j) {
-      long long wp = 0, wv = 0, tp = 0, tv = 0;
-#pragma unroll
-      for (int w = 0; w < kBlock / 32; ++w) {
-        wp += (w < warp) ? s_wc[w][j] : 0;
-        wv += (w < warp) ? s_wl[w][j] : 0;
-        tp += s_wc[w][j];
-        tv += s_wl[w][j];
-      }
+#pragma unroll 1
+    for (int j = 0; j < SUB; ++j) {
       const long long i = tile * kOutTile + (long long)j * kPolyTile + threadIdx.x;
-      const long long pb = bp + wp + s_xc[j][threadIdx.x];
-      const long long vb = bv + wv + s_xl[j][threadIdx.x];
-      bp += tp;
-      bv += tv;
+      const long long at = s_sum[j * kWarps + warp] + s_x[j][threadIdx.x];
+      const long long pb = at >> 33, vb = at & kLen;
       const int pc = s_pc[j][threadIdx.x];
-      const long long l = s_len[j][threadIdx.x];
-      const long long c = pc == 0 ? 1 : pc;
+      const long long l = s_len[j][threadIdx.x], src = s_src[j][threadIdx.x];
       long long sj = -1;
       if (i < n) {
-        if (pb + c > m || vb + l > 3 * m) {
+        if (pb + max(pc, 1) > m || vb + l > 3 * m) {
           set_error(C, POLYLLA_ERR_LIMIT, 80);
         } else {
           if (obase) obase[i] = pb;
-          if (pc == 0) {
-            off[pb] = vb;
-          } else {
-            const long long fb = P.pbase[i];
-            long long acc = 0;
-            for (int r = 0; r < pc; ++r) {
-              off[pb + r] = vb + acc;
-              acc += F.len[fb + r];
-            }
-          }
-          const long long src = s_src[j][threadIdx.x];
+          off[pb] = vb;
           if (src < 0 || src + l > pool.cap) set_error(C, POLYLLA_ERR_LIMIT, 81);
           else sj = src;
         }
       }
-      const unsigned um = __ballot_sync(0xffffffffu, sj >= 0);
-      const long long prev_end = __shfl_up_sync(0xffffffffu, sj + l, 1);
-      const bool first = sj >= 0 && (lane == 0 || !((um >> (lane - 1)) & 1u) || prev_end != sj);
-      unsigned starts = __ballot_sync(0xffffffffu, first);
-      const unsigned breaks = starts | ~um;
-      while (starts) {
-        const int a = __ffs(starts) - 1;
-        starts &= starts - 1;
-        const unsigned above = breaks & ~((2u << a) - 1u);
-        const int e = above ? __ffs(above) - 1 : 32;
-        const long long s0 = __shfl_sync(0xffffffffu, sj, a);
-        const long long d0 = __shfl_sync(0xffffffffu, vb, a);
-        const long long s1 = __shfl_sync(0xffffffffu, sj + l, e - 1);
-        const long long run = s1 - s0;
-        const int* __restrict__ from = pool.v + s0;
-        int* __restrict__ to = vtx + d0;
-        // up to four loads in flight per lane before their stores
-        for (long long k = lane; k < run; k += 128) {
-          int v[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (k + 32 * u < run) v[u] = from[k + 32 * u];
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (k + 32 * u < run) to[k + 32 * u] = v[u];
-        }
+      // the offsets of the further pieces: pieces lie back to back in the pool
+      for (unsigned left = __ballot_sync(0xffffffffu, sj >= 0 && pc > 1); left; left &= left - 1) {
+        const int a = __ffs(left) - 1;
+        const int pa = __shfl_sync(0xffffffffu, pc, a);
+        const long long p0 = __shfl_sync(0xffffffffu, pb, a), v0 = __shfl_sync(0xffffffffu, vb, a);
+        const long long q0 = __shfl_sync(0xffffffffu, sj, a);
+        const long long fb = __shfl_sync(0xffffffffu, (long long)(pc > 1 ? P.pbase[i] : 0), a);
+        for (int r = 1 + lane; r < pa; r += 32) off[p0 + r] = v0 + (F.pos[fb + r] - q0);
       }
+      // the copy: start is the polygon's place in the warp's stretch
+      const long long w0 = __shfl_sync(0xffffffffu, vb, 0);
+      const long long total = __shfl_sync(0xffffffffu, vb + l, 31) - w0;
+      const int E = total <= 3 * m ? (int)total : 0;  // (more only after an error)
+      const int start = (int)(vb - w0);
+      const bool some = l > 0;
+      const unsigned um = __ballot_sync(0xffffffffu, some);
+      if (some)
+        s_dist[warp][__popc(um & ((1u << lane) - 1u))] = sj >= 0 ? sj - start : -(1ll << 40);
+      __syncwarp();
+      const unsigned upto = (2u << lane) - 1u;
+      int* const to = vtx + w0;
+      int before = -1;
+      for (int e0 = 0; e0 < E; e0 += 32 * kOutLoads) {
+        int v[kOutLoads];
+        unsigned ok = 0;
+#pragma unroll
+        for (int u = 0; u < kOutLoads; ++u) {
+          const int wu = e0 + 32 * u;
+          if (wu < E) {
+            const unsigned starts =
+                __reduce_or_sync(0xffffffffu, some && start >> 5 == wu >> 5 ? 1u << (start & 31) : 0u);
+            const long long src = s_dist[warp][before + __popc(starts & upto)] + (wu + lane);
+            before += __popc(starts);
+            if (wu + lane < E && src >= 0) {
+              v[u] = pool.v[src];
+              ok |= 1u << u;
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kOutLoads; ++u)
+          if (ok >> u & 1u) to[e0 + 32 * u + lane] = v[u];
+      }
+      __syncwarp();
     }
     if (s_clear) {  // every tile has finished its look-back
       for (long long q = threadIdx.x; q < ntiles; q += kBlock) status[q] = 0;
@@ -210,9 +214,15 @@ cudaError_t launch_final_write(const DevMesh& M, const int* tf, const PolyArrays
                                const FinalPieces& F, const Pool& pool, unsigned long long* status,
                                long long* off, int* vtx, long long* obase, Counters* C, int grid,
                                cudaStream_t s) {
-  static std::atomic<int> cap{0};
-  grid = resident_grid(reinterpret_cast<const void*>(k_final_write), kBlock, 0, grid, &cap);
-  k_final_write<<<grid, kBlock, 0, s>>>(M, tf, P, F, pool, status, off, vtx, obase, C);
+  // seeds are about a seventh of the triangles, and never more than all of them
+  static std::atomic<int> cap1{0}, cap4{0};
+  if (M.m <= kOutSmall) {
+    grid = resident_grid(reinterpret_cast<const void*>(k_final_write<1>), kBlock, 0, grid, &cap1);
+    k_final_write<1><<<grid, kBlock, 0, s>>>(M, tf, P, F, pool, status, off, vtx, obase, C);
+  } else {
+    grid = resident_grid(reinterpret_cast<const void*>(k_final_write<4>), kBlock, 0, grid, &cap4);
+    k_final_write<4><<<grid, kBlock, 0, s>>>(M, tf, P, F, pool, status, off, vtx, obase, C);
+  }
   return cudaGetLastError();
 }
 

@@ -44,8 +44,8 @@ CASES = {
     "queue-full": lambda: [spiral_wheel(9)] * 32 + [spiral_wheel(9)] * 31 + [spiral_wheel(11)],
     # ten-tip polygons side by side: more tips than a warp's list holds
     "tip-list-overflow": lambda: [tip_hub()] * 6 + [small()],
-    # seed counts about a warp's and a block's
-    **{f"squares-{k}x{k}": (lambda k=k: [grid_mesh(k, seed=k)[0]]) for k in (1, 5, 6, 16, 17)},
+    # seed counts about a warp's, a block's and the output tiles' (256 and 1024)
+    **{f"squares-{k}x{k}": (lambda k=k: [grid_mesh(k, seed=k)[0]]) for k in (1, 5, 6, 16, 17, 32, 33)},
 }
 
 
