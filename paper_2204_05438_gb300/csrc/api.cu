@@ -403,7 +403,7 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
   const int gw = grid_for(h, M.m, kWalkThreads / 2);
   POLY_TRY(launch(h, "walk", s, [&] {
     return launch_walk(M, h->tf, h->entry, h->P, h->pool, h->Lg, h->Dl, h->Dm, h->walk_cap,
-                       repair, M.m < kSmallMeshTri ? 3 : 0, h->C, gw, s, pdl);
+                       repair, M.m < kSmallMeshTri ? kRsMaxSplit + 1 : 0, h->C, gw, s, pdl);
   }));
   // repair_one (this stream), repair_multi and long (side streams) at once
   const bool fork = !h->timing && h->overlap;

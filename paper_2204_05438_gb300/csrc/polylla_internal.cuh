@@ -311,12 +311,14 @@ struct LongList {
 // blocks; with tips_to_long > 0 (small meshes), so do polygons with that many tips
 // or more when `repair` (the block splits their tips in parallel; one thread would
 // split them one after another).
-constexpr long long kSmallMeshTri = 1ll << 16;  // meshes below this: tips_to_long = 3
+constexpr int kRsMaxSplit = 8;  // tips that a warp splits together (k_repair_multi)
+constexpr long long kSmallMeshTri = 1ll << 16;  // meshes below this: more go to blocks
 cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,
                         const Pool& pool, const LongList& Lg, const LongList& D1,
                         const LongList& Dm, int cap, int repair, int tips_to_long, Counters* C,
                         int grid, cudaStream_t s, bool pdl);
-// One thread per polygon with one tip / with several tips (listed by k_walk).
+// One thread per polygon with one tip / one warp per polygon with several tips (listed
+// by k_walk).
 cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
                               const FinalPieces& F, const Pool& pool, const LongList& D1, int rare,
                               Counters* C, int sms, cudaStream_t s, bool pdl);

@@ -12,10 +12,8 @@
 //           left to one thread block (long.cu).
 //   k_repair_one    one thread per polygon with one tip: split it and cut the
 //           two pieces out of the vertex sequence the walk left in the pool.
-//   k_repair_multi  one thread per polygon with several tips: the cycle becomes
-//           a linked list of nodes in shared memory, and each split (smallest tip
-//           of the current piece first) adds two chord nodes and relinks four
-//           pointers.
+//   k_repair_multi  one warp per polygon with several tips: all split edges at once,
+//           then the pieces as the cycles of the new successors.
 // The paper's AtomicAdd on i_Gmesh / i_Gpos is replaced by the output scan
 // (final.cu); the pool order does not matter.
 #include "walk.cuh"
@@ -43,10 +41,6 @@ __device__ __forceinline__ long long warp_alloc(long long* counter, int need) {
 }
 
 
-// Polygons with more tips than this are split by one thread re-walking its pieces
-// (repair_seq); those with 2..kRsMaxSplit tips get the walk's tip records and the
-// several-tip kernel's node list.
-constexpr int kRsMaxSplit = 8;
 
 // The walk of 32 seeds by a warp.  The non-frontier edges of a region form its
 // longest-edge tree (every triangle but the terminal pair hangs from the neighbour
@@ -143,7 +137,7 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
   const int* __restrict__ tri = M.tri;
   const int n = (int)C->n_seeds;  // below 2^29
   const int H = (int)(3 * M.m);
-  // polygons with 2 to this many tips get tip records
+  // polygons with 2 to this many tips leave their half-edges to the several-tip kernel
   const int most_rec = tips_to_long > 0 ? min(tips_to_long - 1, kRsMaxSplit) : kRsMaxSplit;
   unsigned st_len = 0, st_tips = 0, st_tippolys = 0;
   // 32 seeds a warp and round, or fewer while that leaves no warp without any: on a
@@ -407,8 +401,8 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
       // ---- records and lists
       long long roff = off + first;
       if (__any_sync(full, rec)) {
-        // several tips: the sequence and the records (rotated tip index, tip
-        // half-edge) get space of their own, which the pieces overwrite
+        // several tips: the half-edges get space of their own, which the pieces
+        // overwrite
         const long long o = warp_alloc(&C->pool_alloc, rec ? L + 2 * ntips : 0);
         if (rec) roff = o;
       }
@@ -422,7 +416,7 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
         const int pr = __shfl_sync(full, rank, s);
         const long long po = __shfl_sync(full, roff, s);
         for (int q = lane; q < l; q += 32)
-          pool.v[po + (q >= pr ? q - pr : q - pr + l)] = B.u.v[p0 + q];
+          pool.v[po + (q >= pr ? q - pr : q - pr + l)] = B.he[p0 + q];
       }
       if (repair) {
         for (int t0 = 0; t0 < min(tn, kTipSlots); t0 += 32) {
@@ -430,31 +424,22 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
           const bool live = t < min(tn, kTipSlots) && B.tip_h[t] >= 0;
           const int at = live ? B.tip_at[t] : 0;
           const int s = at >> 16, owner = live ? B.lane[s] : 0;
-          const long long po = __shfl_sync(full, roff, owner);
-          const int how = __shfl_sync(full, (int)(split && kept) | (int)rec << 1, owner);
-          if (live && (how & 1)) {
+          const bool listed = __shfl_sync(full, (int)(split && kept), owner) != 0;
+          if (live && listed) {
             const int inf = B.info[s], pr = B.rank[s];
             const int p0 = inf & 1023, l = inf >> 10;
             const int q = at & 0xffff;
             const int b = B.u.v[p0 + (q + 1 < l ? q + 1 : 0)];  // the tip vertex
-            int order = 0;
             bool lowest = true;
             const bool one = B.nt[s] == 1;
             for (int k = 0; k < min(tn, kTipSlots) && !one; ++k) {
               if (B.tip_at[k] >> 16 != s || B.tip_h[k] < 0) continue;
               const int qk = B.tip_at[k] & 0xffff;
-              order += k < t;
               lowest &= B.u.v[p0 + (qk + 1 < l ? qk + 1 : 0)] >= b;
             }
-            const int rot = q >= pr ? q - pr : q - pr + l;
-            const int ip = base + owner;
-            if (how & 2) {
-              pool.v[po + l + 2 * order] = rot;
-              pool.v[po + l + 2 * order + 1] = B.tip_h[t];
-            }
             if (lowest) {
-              P.tip_h[ip] = B.tip_h[t];
-              if (one) P.pbase[ip] = rot;  // the tip's index in the sequence
+              P.tip_h[base + owner] = B.tip_h[t];
+              if (one) P.pbase[base + owner] = q >= pr ? q - pr : q - pr + l;  // its index
             }
           }
         }
@@ -476,7 +461,7 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
           P.start[i] = start;
           P.len[i] = kept ? L : 0;
           P.ntip[i] = ntips;
-          if (ntips > 1) P.pbase[i] = rec ? 1 : 0;  // several tips: records at pos, or none
+          if (ntips > 1) P.pbase[i] = rec ? 1 : 0;  // several tips: half-edges at pos, or none
         }
       }
       __syncwarp();
@@ -734,284 +719,278 @@ __global__ void __launch_bounds__(kBlock) k_repair_one(DevMesh M, uint8_t* lab, 
     atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_splits), (unsigned long long)nd);
 }
 
-// Linked-list reparation of one polygon with several tips per thread.
+// Reparation of one polygon with 2 to kRsMaxSplit tips by a warp.
 //
-// Nodes 0..L-1 are the polygon's frontier half-edges in boundary order from its
-// canonical start (bit 31 set on a barrier-edge tip a->b, i.e. the node followed
-// by twin(a->b)); nodes kWalkCap.. are chord half-edges added by splits.  Each
-// node keeps its half-edge, its origin vertex and next/prev links, all in shared
-// memory, transposed ([node][thread]) so that lanes at the same step hit distinct
-// banks.  The pieces form an ordered list of start nodes, as in repair_seq: the
-// first piece with a tip is split at its smallest tip b (the destination of tip
-// node p) along oj = split_edge(), and is replaced by the piece from oj (b->x)
-// followed by the piece from tw = twin(oj) (x->b).  With q the node of turn(oj)
-// -- the first frontier half-edge after oj around x -- and qp its predecessor:
-//     p -> oj -> q   and   qp -> tw -> next(p),
-// which is the boundary that walking the region with the new frontier edge gives.
-// A split removes the tip at p, and the one at qp if x was a tip, and creates
-// none (x always has a frontier edge of the region besides the chord), so only
-// those two flags change.
+// The walk left the polygon's half-edges in boundary order from its canonical start.
+// A lane per tip finds its split edge from the labels as they are (a tip's fan changes
+// only through a split edge that ends at the tip, which removes it as a tip), and the
+// rule's order -- the first piece with a tip is split at its smallest tip -- comes to
+// all tips in increasing vertex order, leaving out those a smaller tip's split edge
+// ends on.  With the kept split edges marked frontier, the nodes are the polygon's
+// half-edges and two per split edge (oj = b->x and tw = x->b); a node's successor is
+// the next half-edge, unless a split edge ends at its destination: then it is found by
+// turning.  A lane per side of each split edge walks its piece, the piece's smallest
+// such node names it, and the pieces' order is the rule's tree of splits: the two sides
+// of each split joined, the largest tip first, the side of oj on the left.
 //
-// The node list comes from the walk's records (the origins from the canonical
-// start, and each tip's index and half-edge): the other nodes' half-edges stay
-// unknown (kSuccMask) unless needed.  q is the piece's
-// only node with origin x; when x occurs more than once in the piece, q is the
-// one whose successor's origin is dest(turn(oj)) (a directed edge occurs once in
-// a boundary).  A finished piece starts at its smallest vertex; when that vertex
-// occurs more than once, the piece's half-edges are found by turning from a node
-// whose half-edge is known (a chord), and the smallest (origin, half-edge) key
-// decides.  The pieces are written over the records (as long as the polygon and
-// its tip records, at least its final length).
-constexpr int kRsThreads = 64;
+// What bounds it: the chain of dependent loads of one polygon (its records, the fans,
+// the turns), about 17 us; the one-thread form split tip by tip, walking its pieces
+// in between.  Before and after, us: gmm16-10m (19,880 polygons) 71 and 57, 200,000
+// mixture points (416) 65 and 18, where it was the longest of the three kernels that
+// run side by side (the run: 122 and 104).
+constexpr int kRsThreads = 128;
+constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsNodes = kWalkCap + 2 * kRsMaxSplit;
-constexpr int kRsList = kRsMaxSplit + 2;
-constexpr size_t kRsSmem =
-    (size_t)kRsThreads * (kRsNodes * (2 * sizeof(int) + 2) + kRsList);
+constexpr int kRsRounds = (kRsNodes + 31) / 32;
+static_assert(kWalkCap == 64 && kRsNodes < 256 && 2 * kRsMaxSplit <= 32 &&
+                  4 * (kRsMaxSplit + 1) <= 64,
+              "two half-edges a lane, a lane per side, a piece order of 4-bit numbers");
+
+struct SplitBuf {
+  int h[kRsNodes], v[kRsNodes];  // nodes: half-edge, origin
+  int end[2 * kRsMaxSplit];      // the split edges' end vertices
+  unsigned char nx[kRsNodes], todo[kRsNodes];
+  unsigned char tip[kRsMaxSplit];
+  unsigned char pstart[kRsMaxSplit + 1], plen[kRsMaxSplit + 1];
+};
+
+// Returns the number of pieces (their records in F from *foff), or -1; every lane of
+// the warp calls it.  hs: the polygon's L half-edges, overwritten with the pieces.
+__device__ __forceinline__ int split_by_warp(const DevMesh& M, uint8_t* lab, int* tf, SplitBuf& B,
+                                             int L, int nt, int* hs, long long off,
+                                             const FinalPieces& F, int rare, Counters* C,
+                                             long long* foff) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const int H = (int)(3 * M.m);
+  const long long limit = 3 * M.m + 3;
+  bool bad = false;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int q = lane + 32 * r;
+    if (q < L) {
+      const int h = hs[q];
+      bad |= (unsigned)h >= (unsigned)H;
+      B.h[q] = h;
+    }
+  }
+  if (__any_sync(full, bad)) return -1;
+  __syncwarp();
+  // origins, and the tips: half-edges followed by their twins
+  int found = 0;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int q = lane + 32 * r;
+    bool tip = false;
+    if (q < L) {
+      const int h = B.h[q];
+      B.v[q] = M.tri[h];
+      tip = tf_twin(tf[h]) == B.h[q + 1 < L ? q + 1 : 0];
+    }
+    const unsigned t = __ballot_sync(full, tip);
+    const int k = found + __popc(t & lt);
+    if (tip && k < kRsMaxSplit) B.tip[k] = (unsigned char)q;
+    found += __popc(t);
+  }
+  __syncwarp();
+  if (found != nt) return -1;
+  // a lane per tip b: its split edge oj = b->x
+  int b = 0x7fffffff, oj = -1, tw = -1, x = -1;
+  if (lane < nt) {
+    const int q = B.tip[lane];
+    b = B.v[q + 1 < L ? q + 1 : 0];
+    oj = split_edge(tf, B.h[q], H);
+    tw = oj >= 0 ? tf_twin(tf[oj]) : H;
+    if (tw < H) x = M.tri[tw];
+    else bad = true;
+  }
+  if (__any_sync(full, bad)) return -1;
+  // in increasing vertex order; a split edge that ends on a larger tip removes it
+  int rank = 0, hit = -1;
+  for (int k = 0; k < nt; ++k) rank += __shfl_sync(full, b, k) < b;
+  for (int k = 0; k < nt; ++k) {
+    const int bk = __shfl_sync(full, b, k), rk = __shfl_sync(full, rank, k);
+    if (bk == x && bk > b) hit = rk;
+  }
+  unsigned gone = 0;
+  for (int r = 0; r < nt; ++r) {
+    const unsigned at = __ballot_sync(full, lane < nt && rank == r);
+    if (!at) return -1;  // (a vertex twice among the tips: a corrupt mesh)
+    const int to = __shfl_sync(full, hit, __ffs(at) - 1);
+    if (!(gone >> r & 1u) && to >= 0) gone |= 1u << to;
+  }
+  const bool keep = lane < nt && !(gone >> rank & 1u);
+  const int chord = __popc(~gone & ((1u << rank) - 1u));  // among the kept, by vertex
+  const int ns = __popc(__ballot_sync(full, keep)), N = L + 2 * ns;
+  if (keep) {
+    B.h[L + 2 * chord] = oj;
+    B.v[L + 2 * chord] = b;
+    B.h[L + 2 * chord + 1] = tw;
+    B.v[L + 2 * chord + 1] = x;
+    B.end[2 * chord] = b;
+    B.end[2 * chord + 1] = x;
+    set_frontier(lab, tf, oj);
+    set_frontier(lab, tf, tw);
+  }
+  __syncwarp();
+  // successors: the next half-edge, or by turning where a split edge ends
+  int ntodo = 0;
+#pragma unroll
+  for (int r = 0; r < kRsRounds; ++r) {
+    const int a = lane + 32 * r;
+    bool turn = a >= L && a < N;
+    if (a < L) {
+      const int nx = a + 1 < L ? a + 1 : 0;
+      const int d = B.v[nx];
+      B.nx[a] = (unsigned char)nx;
+      turn = rare != 0;
+      for (int k = 0; k < 2 * ns; ++k) turn |= B.end[k] == d;
+    }
+    const unsigned t = __ballot_sync(full, turn);
+    if (turn) B.todo[ntodo + __popc(t & lt)] = (unsigned char)a;
+    ntodo += __popc(t);
+  }
+  __syncwarp();
+  for (int t = lane; t < ntodo; t += 32) {
+    const int a = B.todo[t];
+    long long steps = 0;
+    const int g = turn_tf(tf, B.h[a], H, steps, limit);
+    int c = 0;
+    while (c < N && B.h[c] != g) ++c;
+    if (g < 0 || c == N) bad = true;
+    else B.nx[a] = (unsigned char)c;
+  }
+  if (__any_sync(full, bad)) return -1;
+  __syncwarp();
+  // a lane per side of each split edge walks its piece
+  const bool side = lane < 2 * ns;
+  int name = 255, len = 0, least = 0x7fffffff, start = 0;
+  if (side) {
+    int a = L + lane;
+    do {
+      const int o = B.v[a];
+      if (o < least || (o == least && B.h[a] < B.h[start])) {
+        least = o;
+        start = a;
+      }
+      if (a >= L && a < name) name = a;
+      a = B.nx[a];
+    } while (++len <= N && a != L + lane);
+    bad = len > N;
+  }
+  if (__any_sync(full, bad)) return -1;
+  const unsigned owners = __ballot_sync(full, side && name == L + lane);
+  const int np = __popc(owners);
+  if (np != ns + 1) return -1;
+  // the piece of each side, numbered by name; each piece's start and length
+  const int piece = side ? __popc(owners & ((1u << (name - L)) - 1u)) : 0;
+  if (owners >> lane & 1u) {
+    B.pstart[piece] = (unsigned char)start;
+    B.plen[piece] = (unsigned char)len;
+  }
+  __syncwarp();
+  // the tree of splits: lane p holds the group of piece p and, as a group's first
+  // piece, the group's pieces in order (4 bits each) and their number
+  int group = lane, count = 1;
+  unsigned long long order = (unsigned)lane & 15u;
+  for (int k = ns - 1; k >= 0; --k) {
+    const int ga = __shfl_sync(full, group, __shfl_sync(full, piece, 2 * k));
+    const int gb = __shfl_sync(full, group, __shfl_sync(full, piece, 2 * k + 1));
+    if (ga == gb) return -1;
+    const unsigned long long ob = __shfl_sync(full, order, gb);
+    const int cb = __shfl_sync(full, count, gb);
+    if (lane == ga) {
+      order |= ob << (4 * count);
+      count += cb;
+    }
+    if (group == gb) group = ga;
+  }
+  order = __shfl_sync(full, order, __shfl_sync(full, group, 0));
+  // the pieces, a lane each, from their canonical starts
+  const int p = lane < np ? (int)(order >> (4 * lane) & 15u) : 0;
+  const int l = lane < np ? B.plen[p] : 0;
+  int at = l;
+#pragma unroll
+  for (int d = 1; d < 16; d <<= 1) {
+    const int y = __shfl_up_sync(full, at, d);
+    if (lane >= d) at += y;
+  }
+  at -= l;
+  long long f = 0;
+  if (lane == 0)
+    f = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->fslot_alloc),
+                             (unsigned long long)np);
+  f = __shfl_sync(full, f, 0);
+  if (f + np > F.cap) return -1;
+  if (lane < np) {
+    F.pos[f + lane] = off + at;
+    F.len[f + lane] = l;
+    int a = B.pstart[p];
+    for (int k = 0; k < l; ++k) {
+      hs[at + k] = B.v[a];
+      a = B.nx[a];
+    }
+  }
+  *foff = f;
+  return np;
+}
 
 __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t* lab, int* tf,
                                                              PolyArrays P, FinalPieces F,
                                                              Pool pool, LongList Dm, int rare,
                                                              Counters* C) {
-  extern __shared__ int rs_smem[];
-  int* nh = rs_smem;                                   // [kRsNodes][kRsThreads]
-  int* no = nh + kRsNodes * kRsThreads;                // origins
-  uint8_t* nx = reinterpret_cast<uint8_t*>(no + kRsNodes * kRsThreads);
-  uint8_t* pv = nx + kRsNodes * kRsThreads;
-  uint8_t* ps = pv + kRsNodes * kRsThreads;            // [kRsList][kRsThreads]
-  const int t = threadIdx.x;
-#define NH(j) nh[(j) * kRsThreads + t]
-#define NO(j) no[(j) * kRsThreads + t]
-#define NX(j) nx[(j) * kRsThreads + t]
-#define PV(j) pv[(j) * kRsThreads + t]
-#define PS(j) ps[(j) * kRsThreads + t]
+  __shared__ SplitBuf s_buf[kRsWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long nd = min(C->n_multi, Dm.cap);
   const int H = (int)(3 * M.m);
   const long long limit = 3 * M.m + 3;
   unsigned st_splits = 0, st_seq = 0, st_turn = 0;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < nd;
-       base += (long long)gridDim.x * blockDim.x) {
-    const long long d = base + t;
-    const long long i = (d < nd) ? Dm.poly[d] : -1;
-    const int L = (i >= 0) ? P.len[i] : 0;
-    const int nt = (i >= 0) ? P.ntip[i] : 0;
-    const bool listed = nt <= kRsMaxSplit && L <= kWalkCap;
-    const bool rec = i >= 0 && listed && nt >= 2 && L >= 3 && P.pbase[i] == 1;
-    const long long off0 = warp_alloc(&C->pool_alloc, i >= 0 && !rec ? L + 2 * nt : 0);
-    const long long foff = warp_alloc(&C->fslot_alloc, i >= 0 ? nt + 1 : 0);
-    if (i < 0) continue;
-    const long long off = rec ? P.pos[i] : off0;
-    if (L < 3 || off < 0 || off + L + 2 * nt > pool.cap || foff + nt + 1 > F.cap) {
-      set_error(C, POLYLLA_ERR_LIMIT, 56);
-      continue;
+  for (long long d = (long long)blockIdx.x * kRsWarps + warp; d < nd;
+       d += (long long)gridDim.x * kRsWarps) {
+    const int i = Dm.poly[d];
+    const int L = P.len[i], nt = P.ntip[i];
+    int cnt = -1;
+    long long foff = 0;
+    if (nt >= 2 && nt <= kRsMaxSplit && L >= 3 && L <= kWalkCap && P.pbase[i] == 1) {
+      const long long off = P.pos[i];
+      if (off >= 0 && off + L + 2 * nt <= pool.cap)
+        cnt = split_by_warp(M, lab, tf, s_buf[warp], L, nt, pool.v + off, off, F, rare, C, &foff);
+      if (rare && cnt > 0) st_turn += cnt;
+    } else if (nt > kRsMaxSplit && L >= 3) {
+      if (lane == 0) {  // more tips than the nodes hold: one thread, piece by piece
+        ++st_seq;
+        const long long off = (long long)atomicAdd(
+            reinterpret_cast<unsigned long long*>(&C->pool_alloc), (unsigned long long)(L + 2 * nt));
+        foff = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->fslot_alloc),
+                                    (unsigned long long)(nt + 1));
+        if (off + L + 2 * nt <= pool.cap && foff + nt + 1 <= F.cap) {
+          const Cyc first{P.start[i], L, P.tip_h[i], nt, true};
+          cnt = repair_seq(M.tri, tf, lab, first, nt + 1, H, limit, F.h + foff, F.pos + foff,
+                           F.len + foff, pool.v + off, off, L + 2 * nt);
+        }
+      }
     }
-    int cnt;
-    if (!listed) {
-      ++st_seq;
-      const Cyc first{P.start[i], L, P.tip_h[i], nt, true};
-      cnt = repair_seq(M.tri, tf, lab, first, nt + 1, H, limit, F.h + foff, F.pos + foff,
-                       F.len + foff, pool.v + off, off, L + 2 * nt);
-    } else {
-      cnt = -1;
-      bool bad = false;
-      if (!rec) {
-        bad = true;  // the walk leaves records for every such polygon
+    if (lane == 0) {
+      if (cnt < 0) {
+        set_error(C, POLYLLA_ERR_LIMIT, 54);
       } else {
-        const int* rv = pool.v + off;
-        for (int j0 = 0; j0 < L; j0 += kSeqChunk) {
-          int w[kSeqChunk];
-#pragma unroll
-          for (int k = 0; k < kSeqChunk; ++k) w[k] = (j0 + k < L) ? rv[j0 + k] : 0;
-#pragma unroll
-          for (int k = 0; k < kSeqChunk; ++k) {
-            const int j = j0 + k;
-            if (j >= L) break;
-            NH(j) = kSuccMask;
-            NO(j) = w[k];
-            NX(j) = (uint8_t)(j + 1 == L ? 0 : j + 1);
-            PV(j) = (uint8_t)(j == 0 ? L - 1 : j - 1);
-          }
-        }
-        for (int k = 0; k < nt; ++k) {
-          const int ix = rv[L + 2 * k], hh = rv[L + 2 * k + 1];
-          if ((unsigned)ix >= (unsigned)L || (unsigned)hh >= (unsigned)H) {
-            bad = true;
-            break;
-          }
-          NH(ix) = hh | kTipFlag;
-        }
+        P.pcnt[i] = cnt;
+        P.pbase[i] = (int)foff;
+        P.flen[i] = L + 2 * (cnt - 1);
+        st_splits += cnt - 1;
       }
-      int nn = kWalkCap;  // next chord node
-      int count = 1;
-      PS(0) = 0;
-      long long acc = 0;
-      int j = 0;
-      while (!bad && j < count) {
-        const int s0 = PS(j);
-        // the piece: its smallest tip, its smallest vertex and how often it occurs
-        int tb = 0x7fffffff, tipn = -1, mo = 0x7fffffff, mn = s0, mc = 0, len = 0;
-        int v = s0;
-        do {
-          const int x = NH(v);
-          const int nv = NX(v);
-          if (x < 0) {
-            const int b = NO(nv);
-            if (b < tb) {
-              tb = b;
-              tipn = v;
-            }
-          }
-          const int o = NO(v);
-          if (o < mo) {
-            mo = o;
-            mn = v;
-            mc = 1;
-          } else if (o == mo) {
-            ++mc;
-          }
-          ++len;
-          v = nv;
-        } while (v != s0 && len <= kRsNodes);
-        if (len > kRsNodes) {
-          bad = true;
-          break;
-        }
-        if (tipn < 0) {  // finished piece: its origins from the canonical start
-          if (mc > 1 || rare) {  // the smallest vertex repeats: compare (origin, half-edge)
-            ++st_turn;
-            int c0 = -1;
-            v = s0;
-            for (int k = 0; k < len && c0 < 0; ++k, v = NX(v))
-              if ((NH(v) & kSuccMask) != kSuccMask) c0 = v;
-            if (c0 < 0) {
-              bad = true;
-              break;
-            }
-            v = c0;
-            for (int k = 0; k + 1 < len && !bad; ++k) {  // unknown half-edges by turning
-              const int nv = NX(v);
-              if ((NH(nv) & kSuccMask) == kSuccMask) {
-                long long steps = 0;
-                const int g = turn_tf(tf, NH(v) & kSuccMask, H, steps, limit);
-                if (g < 0) bad = true;
-                else NH(nv) = g;
-              }
-              v = nv;
-            }
-            if (bad) break;
-            unsigned long long best = ~0ull;
-            v = s0;
-            for (int k = 0; k < len; ++k, v = NX(v)) {
-              const unsigned long long key = vkey(NO(v), NH(v) & kSuccMask);
-              if (key < best) {
-                best = key;
-                mn = v;
-              }
-            }
-          }
-          int* out = pool.v + off + acc;
-          v = mn;
-          for (int k = 0; k < len; ++k) {
-            out[k] = NO(v);
-            v = NX(v);
-          }
-          F.pos[foff + j] = off + acc;
-          F.len[foff + j] = len;
-          acc += len;
-          ++j;
-          continue;
-        }
-        if (count + 1 > nt + 1 || nn + 2 > kRsNodes) {
-          bad = true;
-          break;
-        }
-        const int oj = split_edge(tf, NH(tipn) & kSuccMask, H);
-        if (oj < 0) {
-          bad = true;
-          break;
-        }
-        const int tw = tf_twin(tf[oj]);
-        if (tw >= H) {
-          bad = true;
-          break;
-        }
-        set_frontier(lab, tf, oj);
-        set_frontier(lab, tf, tw);
-        const int x = M.tri[tw];  // origin of tw = dest(oj)
-        // q: the piece's node leaving x at turn(oj)
-        int q = -1, nq = 0;
-        v = s0;
-        for (int k = 0; k < len; ++k, v = NX(v)) {
-          if (NO(v) == x) {
-            q = v;
-            ++nq;
-          }
-        }
-        if (nq != 1 || rare) {  // x repeats: the node whose edge is x -> dest(turn(oj))
-          long long steps = 0;
-          const int g = turn_tf(tf, oj, H, steps, limit);
-          if (g < 0 || g == tw) {
-            bad = true;
-            break;
-          }
-          const int y = M.tri[he_next(g)];
-          q = -1;
-          v = s0;
-          for (int k = 0; k < len; ++k, v = NX(v))
-            if (NO(v) == x && NO(NX(v)) == y) q = v;
-          if (q < 0) {
-            bad = true;
-            break;
-          }
-          if ((NH(q) & kSuccMask) == kSuccMask) NH(q) = g;
-        }
-        const int qp = PV(q);
-        const int pn = NX(tipn);
-        const int u = nn, w = nn + 1;
-        nn += 2;
-        NH(u) = oj;
-        NO(u) = tb;
-        NH(w) = tw;
-        NO(w) = x;
-        NX(tipn) = (uint8_t)u;
-        PV(u) = (uint8_t)tipn;
-        NX(u) = (uint8_t)q;
-        PV(q) = (uint8_t)u;
-        NX(qp) = (uint8_t)w;
-        PV(w) = (uint8_t)qp;
-        NX(w) = (uint8_t)pn;
-        PV(pn) = (uint8_t)w;
-        NH(tipn) &= kSuccMask;
-        NH(qp) &= kSuccMask;
-        for (int k = count; k > j + 1; --k) PS(k) = PS(k - 1);
-        PS(j) = (uint8_t)u;
-        PS(j + 1) = (uint8_t)w;
-        ++count;
-      }
-      if (!bad) cnt = count;
     }
-#undef NH
-#undef NO
-#undef NX
-#undef PV
-#undef PS
-    if (cnt < 0) {
-      set_error(C, POLYLLA_ERR_LIMIT, 54);
-      continue;
-    }
-    P.pcnt[i] = cnt;
-    P.pbase[i] = (int)foff;
-    P.flen[i] = L + 2 * (cnt - 1);
-    st_splits += cnt - 1;
+    __syncwarp();
   }
-  st_splits = __reduce_add_sync(0xffffffffu, st_splits);
-  st_seq = __reduce_add_sync(0xffffffffu, st_seq);
-  if ((threadIdx.x & 31) == 0 && st_splits)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_splits), (unsigned long long)st_splits);
-  if ((threadIdx.x & 31) == 0 && st_seq)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_seq), (unsigned long long)st_seq);
-  st_turn = __reduce_add_sync(0xffffffffu, st_turn);
-  if ((threadIdx.x & 31) == 0 && st_turn)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_turn), (unsigned long long)st_turn);
+  if (lane == 0) {
+    if (st_splits)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_splits), (unsigned long long)st_splits);
+    if (st_seq)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_seq), (unsigned long long)st_seq);
+    if (st_turn)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_turn), (unsigned long long)st_turn);
+  }
 }
 
 cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
@@ -1028,13 +1007,10 @@ cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const P
                                 const FinalPieces& F, const Pool& pool,
                                 const LongList& Dm, int rare, Counters* C, int sms,
                                 cudaStream_t s) {
-  static std::atomic<bool> attr[kMaxDevices];
-  const cudaError_t e =
-      smem_limit_once(reinterpret_cast<const void*>(k_repair_multi), (int)kRsSmem, attr);
-  if (e != cudaSuccess) return e;
-  const int per_sm = (int)((220 * 1024) / (kRsSmem + 1024));
-  const int grid = sms * (per_sm < 1 ? 1 : per_sm);
-  k_repair_multi<<<grid, kRsThreads, kRsSmem, s>>>(M, lab, tf, P, F, pool, Dm, rare, C);
+  static std::atomic<int> cap{0};
+  const int grid = resident_grid(reinterpret_cast<const void*>(k_repair_multi), kRsThreads, 0,
+                                 (long long)sms * 16, &cap);
+  k_repair_multi<<<grid, kRsThreads, 0, s>>>(M, lab, tf, P, F, pool, Dm, rare, C);
   return cudaGetLastError();
 }
 

@@ -12,7 +12,7 @@ import pytest
 
 import meshgen
 import oracle
-from meshlib import disjoint_union, grid_mesh, spiral_wheel, tip_hub
+from meshlib import disjoint_union, grid_mesh, spiral_wheel, tip_hub, tip_order_meshes
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -121,3 +121,28 @@ def test_polygons_handed_between_blocks_count_once():
         B.all_polygons()
         assert B.stats()["n_vtx_trav"] == want, f"schedule {k}"
     B.close()
+
+
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("rare", [False, True])
+def test_several_tip_polygons(big, rare):
+    """Polygons of 2 to 8 tips, split by a warp: mixture meshes (above 2^16 triangles and
+    below), the meshes on which the order of the tips matters, and hubs with more tips
+    than a warp takes; with every successor found by turning when `rare`."""
+    meshes = tip_order_meshes() + [tip_hub(), meshgen.generate("gmm", 40_000 if big else 8_000,
+                                                                1 << 22, 51)]
+    mesh = side_by_side([m["mesh"] if "mesh" in m else m for m in meshes])
+    ref = oracle.run(mesh)
+    M = pg.from_numpy(mesh)
+    M.set_one_block(0)
+    pg.debug_rare_paths(M.handle, rare)
+    M.run()
+    off, vtx = (t.cpu().numpy() for t in M.polygons())
+    lab = M.labels().cpu().numpy()
+    st = M.stats()
+    M.close()
+    np.testing.assert_array_equal(off, ref["off"])
+    np.testing.assert_array_equal(vtx, ref["vtx"])
+    np.testing.assert_array_equal((lab[:, None] >> np.arange(2, 5)) & 1,
+                                  ref["frontier"].reshape(-1, 3))
+    assert st["n_multi_tip"] > 20 and st["n_splits"] == ref["splits"]
