@@ -274,14 +274,18 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->vtx_final, 3 * m);
   ALLOC(h->C, 1);
 #undef ALLOC
-  // stamped arrays start empty (run stamps are never 0)
-  if (e == cudaSuccess) e = cudaMemset(h->vstamp, 0, sizeof(int) * (size_t)n);
-  // look-back words start zero (each pass leaves them zero)
+  // stamped arrays start empty (run stamps are never 0); look-back words start zero
+  // (each pass leaves them zero).  The clears are waited for: the caller's first run
+  // may be on any stream, and a clear that came late would take words from under it
+  cudaStream_t s0 = h->side[0];
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->vstamp, 0, sizeof(int) * (size_t)n, s0);
   if (e == cudaSuccess)
-    e = cudaMemset(h->seed_status, 0, sizeof(unsigned long long) * (size_t)(seed_tiles(m) + 1));
+    e = cudaMemsetAsync(h->seed_status, 0,
+                        sizeof(unsigned long long) * (size_t)(seed_tiles(m) + 1), s0);
   if (e == cudaSuccess)
-    e = cudaMemset(h->out_status, 0, sizeof(unsigned long long) * (size_t)(ntiles + 1));
-  if (e == cudaSuccess) e = cudaMemset(h->C, 0, sizeof(Counters));
+    e = cudaMemsetAsync(h->out_status, 0, sizeof(unsigned long long) * (size_t)(ntiles + 1), s0);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->C, 0, sizeof(Counters), s0);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s0);
   return cuda_status(e);
 }
 
