@@ -38,8 +38,8 @@ __device__ __forceinline__ void out_counts(const PolyArrays& P, long long i, lon
 // offsets come from a look-back over `status` in the same pass (tiles in ticket
 // order; one word per tile packs the piece count << 33 | vertex count, exact
 // within the mesh size limits), and the last tile writes the totals and the CSR
-// end marker.  The status words clean themselves: the block that completes the
-// last look-back (C->out_done counts them) clears them and the count.
+// end marker.  The status words clean themselves: the block that finishes the last
+// tile (C->out_done counts them) clears them and the count.
 constexpr int kOutLoads = 6;
 constexpr long long kOutSmall = 1ll << 21;  // triangles: 1,230 tiles of 256 polygons
 
@@ -95,7 +95,17 @@ __global__ void __launch_bounds__(kBlock, SUB == 4 ? 6 : 5) k_final_write(DevMes
 #pragma unroll
     for (int j = 0; j < SUB; ++j) {
       const long long i = tile * kOutTile + (long long)j * kPolyTile + threadIdx.x;
-      const long long src = i < n ? (pcj[j] == 0 ? P.pos[i] : F.pos[P.pbase[i]]) : -1;
+      long long src = -1;
+      if (i < n) {
+        if (pcj[j] == 0) {
+          src = P.pos[i];
+        } else {
+          const long long fb = P.pbase[i];
+          if (pcj[j] > 0 && fb >= 0 && fb + pcj[j] <= F.cap) src = F.pos[fb];
+          else pcj[j] = lj[j] = 0;  // (reported with the polygon's missing source)
+        }
+        if (lj[j] < 0) lj[j] = 0;
+      }
       s_src[j][threadIdx.x] = src;
       s_len[j][threadIdx.x] = lj[j];
       s_pc[j][threadIdx.x] = pcj[j];
@@ -124,18 +134,12 @@ __global__ void __launch_bounds__(kBlock, SUB == 4 ? 6 : 5) k_final_write(DevMes
       const long long all = __shfl_sync(0xffffffffu, x, 31);
       const long long ex = lookback_warp(status, tile, all, C);
       if (lane < SUB * kWarps) s_sum[lane] = ex + x - own;
-      if (lane == 0) {
-        // the last look-back to complete clears the status words for the next pass
-        const unsigned long long done =
-            atomicAdd(reinterpret_cast<unsigned long long*>(&C->out_done), 1ull);
-        s_clear = done == (unsigned long long)(ntiles - 1);
-        if (tile == ntiles - 1) {
-          const long long np = (ex + all) >> 33, nv = (ex + all) & kLen;
-          C->n_poly = np;
-          C->n_vtx = nv;
-          if (np <= m) off[np] = nv;
-          else set_error(C, POLYLLA_ERR_LIMIT, 82);
-        }
+      if (lane == 0 && tile == ntiles - 1) {
+        const long long np = (ex + all) >> 33, nv = (ex + all) & kLen;
+        C->n_poly = np;
+        C->n_vtx = nv;
+        if (np <= m) off[np] = nv;
+        else set_error(C, POLYLLA_ERR_LIMIT, 82);
       }
     }
     __syncthreads();
@@ -202,11 +206,19 @@ __global__ void __launch_bounds__(kBlock, SUB == 4 ? 6 : 5) k_final_write(DevMes
       }
       __syncwarp();
     }
-    if (s_clear) {  // every tile has finished its look-back
+    if (threadIdx.x == 0) {
+      // the last tile to finish clears the status words for the next pass; the fence
+      // keeps this tile's own word from arriving after that
+      __threadfence();
+      const unsigned long long done =
+          atomicAdd(reinterpret_cast<unsigned long long*>(&C->out_done), 1ull);
+      s_clear = done == (unsigned long long)(ntiles - 1);
+    }
+    __syncthreads();
+    if (s_clear) {
       for (long long q = threadIdx.x; q < ntiles; q += kBlock) status[q] = 0;
       if (threadIdx.x == 0) C->out_done = 0;
     }
-    __syncthreads();
   }
 }
 

@@ -250,7 +250,7 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // gets the tile's offset by a decoupled look-back over `status` (one word per
 // tile), and writes each sub-tile's seeds -- staged in shared memory -- coalesced.
 // The last tile writes the seed count to C->n_seeds.  The status words clean
-// themselves: the block that completes the last look-back (C->seed_done counts
+// themselves: the block that finishes the last tile (C->seed_done counts
 // them) clears them and the count, so nothing has to be zeroed before the next
 // run; the ticket counter C->seed_ticket starts at zero with the label phase's
 // counters.
@@ -344,10 +344,6 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
       if (lane == 0) {
         s_base = ex;
         if (bt == nbt - 1) C->n_seeds = ex + total;
-        // the last look-back to complete clears the status words for the next run
-        const unsigned long long done =
-            atomicAdd(reinterpret_cast<unsigned long long*>(&C->seed_done), 1ull);
-        s_clear = done == (unsigned long long)(nbt - 1);
       }
     }
     __syncthreads();
@@ -377,11 +373,19 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
       base += sub_total[j];
       __syncthreads();
     }
-    if (s_clear) {  // every tile has finished its look-back
+    if (threadIdx.x == 0) {
+      // the last tile to finish clears the status words for the next run; the fence
+      // keeps this tile's own word from arriving after that
+      __threadfence();
+      const unsigned long long done =
+          atomicAdd(reinterpret_cast<unsigned long long*>(&C->seed_done), 1ull);
+      s_clear = done == (unsigned long long)(nbt - 1);
+    }
+    __syncthreads();
+    if (s_clear) {
       for (long long q = threadIdx.x; q < nbt; q += kBlock) status[q] = 0;
       if (threadIdx.x == 0) C->seed_done = 0;
     }
-    __syncthreads();
   }
 }
 

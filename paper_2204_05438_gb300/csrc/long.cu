@@ -262,6 +262,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
   for (long long j = blockIdx.x; j < nl; j += gridDim.x) {
     const long long i = Lg.poly[j];
     const int t0 = seeds[i];
+    if (t0 < 0 || t0 >= M.m) {  // (the same for the whole block)
+      if (threadIdx.x == 0) set_error(C, POLYLLA_ERR_LIMIT, 115);
+      continue;
+    }
     // ---- 1. the region's triangles, by a breadth-first search down its
     //         longest-edge tree: every non-frontier edge is the longest edge of one
     //         of its triangles, and every triangle but the seed's terminal pair hangs

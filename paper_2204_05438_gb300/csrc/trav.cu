@@ -150,7 +150,11 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
   int n1 = 0, nm = 0;  // entries of the warp's list buffers
   for (int base = ((int)blockIdx.x * kWalkWarps + warp) * per; base < n; base += warps * per) {
     const int i = base + lane;
-    const int e0 = lane < per && i < n ? __ldg(entry + i) : -1;
+    int e0 = lane < per && i < n ? __ldg(entry + i) : -1;
+    if (e0 >= H) {  // (no seed pass writes one)
+      set_error(C, POLYLLA_ERR_LIMIT, 51);
+      e0 = -1;
+    }
     int x0 = e0 >= 0 ? __ldg(tf + e0) : -1;
     bool big = false;  // too long for a walk: left to a thread block
     for (int b0 = 0; b0 < per && base + b0 < n;) {
