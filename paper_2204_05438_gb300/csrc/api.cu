@@ -42,9 +42,7 @@ struct polylla_mesh {
   int sms = 148;
   bool owns_inputs = false;
   bool owns_twin = false;      // twin built on the device (handle-owned)
-  int* tw_cnt = nullptr;       // twin construction scratch: per-vertex counts,
-  int* tw_start = nullptr;     // first slots (n + 1),
-  int2* tw_adj = nullptr;      // outgoing half-edges with their destinations (3m)
+  int* tw_table = nullptr;     // twin construction scratch: the table of half-edges
   int phase = kCreated;
   int latest_csr = -1;  // 0: traversal CSR, 1: final CSR
   cudaStream_t last_stream = nullptr;
@@ -67,8 +65,6 @@ struct polylla_mesh {
   LongList Dm{};          // polygons with several tips
   LongList Lg2{};         // long polygons the small blocks hand to the large ones
   int epoch = 0;
-  long long* tile_sum = nullptr;  // twin construction: per-tile counts and offsets
-  long long* tile_off = nullptr;
   unsigned long long* seed_status = nullptr;  // look-back words of the seed pass
   unsigned long long* out_status = nullptr;   // look-back words of the output pass
   long long* off_trav = nullptr;
@@ -183,7 +179,7 @@ void free_all(polylla_mesh* h) {
                   h->loc,      h->vstamp,    h->Lg.poly,   h->P.start,    h->P.len,
                   h->P.ntip,   h->P.pcnt,    h->P.pbase,    h->P.flen,
                   h->P.pos,    h->F.pos,     h->F.len,     h->F.h,        h->pool.v,
-                  h->tile_sum, h->tile_off,  h->off_trav,  h->vtx_trav,   h->off_final,
+                  h->off_trav,  h->vtx_trav,   h->off_final,
                   h->seed_status, h->out_status,
                   h->vtx_final, h->C,         h->Dl.poly,   h->P.tip_h,
                   h->Dm.poly,   h->entry,     h->Lg2.poly,
@@ -191,8 +187,7 @@ void free_all(polylla_mesh* h) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->owns_twin && !h->owns_inputs) cudaFree(const_cast<int*>(h->M.twin));
-  for (void* p : {(void*)h->tw_cnt, (void*)h->tw_start, (void*)h->tw_adj})
-    if (p) cudaFree(p);
+  if (h->tw_table) cudaFree(h->tw_table);
   if (h->owns_inputs) {
     cudaFree(const_cast<long long*>(h->M.xy));
     cudaFree(const_cast<int*>(h->M.tri));
@@ -266,8 +261,6 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->F.len, h->F.cap);
   ALLOC(h->F.h, h->F.cap);
   ALLOC(h->pool.v, h->pool.cap);
-  ALLOC(h->tile_sum, 2 * ntiles);
-  ALLOC(h->tile_off, 2 * ntiles);
   ALLOC(h->seed_status, seed_tiles(m) + 1);
   ALLOC(h->out_status, ntiles + 1);
   ALLOC(h->off_trav, m + 1);
@@ -329,8 +322,6 @@ long long derived_bytes(long long n, long long m) {
   COUNT(c.F.len, c.F.cap);
   COUNT(c.F.h, c.F.cap);
   COUNT(c.pool.v, c.pool.cap);
-  COUNT(c.tile_sum, 2 * ntiles);
-  COUNT(c.tile_off, 2 * ntiles);
   COUNT(c.seed_status, seed_tiles(m) + 1);
   COUNT(c.out_status, ntiles + 1);
   COUNT(c.off_trav, m + 1);
@@ -490,22 +481,20 @@ polylla_status do_repair(polylla_mesh* h, cudaStream_t s) {
 // Scratch of the twin construction, for handles that may build their twin.
 polylla_status alloc_twin_scratch(polylla_mesh* h) {
   const long long m = h->M.m, n = h->M.n;
-  const long long have = (m + kPolyTile - 1) / kPolyTile;  // tile words allocated
-  if ((n + kTriTile - 1) / kTriTile > have) return POLYLLA_ERR_INVALID_ARG;
-  cudaError_t e = dalloc(&h->tw_cnt, n);
-  if (e == cudaSuccess) e = dalloc(&h->tw_start, n + 1);
-  if (e == cudaSuccess) e = dalloc(&h->tw_adj, 3 * m);
-  return cuda_status(e);
+  // far more vertices than triangles (four and more each) are refused
+  if ((n + kTriTile - 1) / kTriTile > (m + kPolyTile - 1) / kPolyTile)
+    return POLYLLA_ERR_INVALID_ARG;
+  return cuda_status(dalloc(&h->tw_table, twin_words(m)));
 }
 
 polylla_status do_build_twin(polylla_mesh* h, cudaStream_t s) {
-  if (!h->tw_adj || !(h->owns_twin || h->owns_inputs)) return POLYLLA_ERR_STATE;
+  if (!h->tw_table || !(h->owns_twin || h->owns_inputs)) return POLYLLA_ERR_STATE;
   h->phase = kCreated;
   h->latest_csr = -1;
   h->lepp_valid = false;
   return launch(h, "build_twin", s, [&] {
-    return launch_build_twin(h->M.tri, h->M.m, h->M.n, const_cast<int*>(h->M.twin), h->tw_cnt,
-                             h->tw_start, h->tw_adj, h->tile_sum, h->tile_off, h->C, h->sms, s);
+    return launch_build_twin(h->M.tri, h->M.m, h->M.n, const_cast<int*>(h->M.twin), h->tw_table,
+                             h->C, s);
   });
 }
 

@@ -26,7 +26,6 @@ constexpr long long kMaxVertices = 1ll << 30;
 constexpr int kWalkThreads = 256;  // k_walk block
 constexpr int kWalkCap = 64;       // longer polygons go to one thread block each (long.cu)
 constexpr int kPolyTile = kBlock;              // per-polygon scans: one polygon per thread
-constexpr int kScanThreads = 1024;
 
 // Device-resident counters of one pipeline run (zeroed by the label phase).
 struct Counters {
@@ -52,8 +51,7 @@ struct Counters {
   long long seed_ticket;  // tile tickets of the seed compaction's look-back
   long long seed_done;    // its completed look-backs (the last one clears the status)
   long long out_done;     // the output pass's completed look-backs (likewise)
-  long long scratch0;     // scan totals that are not reported
-  long long scratch1;
+  long long scratch0;     // split scratch of the one-block path
   long long n_block;      // polygons meshed by the one-block path (block.cu)
   int error;              // first device error (polylla_status), 0 if none
   int err_info;
@@ -165,13 +163,6 @@ __device__ __forceinline__ long long lookback_warp(unsigned long long* status, l
   return excl;
 }
 
-template <typename T>
-__device__ __forceinline__ T block_sum(T v, T* sh) {
-  T tot;
-  block_exclusive_scan(v, &tot, sh);
-  return tot;
-}
-
 // ---------------------------------------------- programmatic dependent launch
 // The kernels of the chain label_max -> label_class -> seed_write -> walk
 // run back to back on one stream.  A chain kernel may be launched with
@@ -261,14 +252,6 @@ cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long lon
                               int* seeds, int* entry, Counters* C, int grid, cudaStream_t s,
                               bool pdl);
 long long seed_tiles(long long m);
-// Exclusive scan of per-tile pairs.  Tile count = ceil(n / tile) with n = *n_dev if
-// n_dev, else n_host.  Totals go to *tot0, *tot1.  end_mode 1: end[n] = total0;
-// end_mode 2: end[total0] = total1 (index checked against end_cap).
-// n_bound: an upper bound of the element count (n_host, or *n_dev on the device).
-cudaError_t launch_scan_tiles(const long long* tile_sum, long long* tile_off, long long n_host,
-                              const long long* n_dev, long long n_bound, int tile,
-                              long long* tot0, long long* tot1, long long* end, int end_mode,
-                              long long end_cap, Counters* C, cudaStream_t s);
 // Per polygon of the traversal (index = seed order), capacity m.
 struct PolyArrays {
   int* start;     // canonical start half-edge of the traversal polygon
@@ -344,10 +327,10 @@ cudaError_t launch_final_write(const DevMesh& M, const int* tf, const PolyArrays
                                const FinalPieces& F, const Pool& pool, unsigned long long* status,
                                long long* off, int* vtx, long long* obase, Counters* C, int grid,
                                cudaStream_t s);
-// The twin array from tri (scratch: cnt n, start n + 1, adj 3m pairs; the tile words).
-cudaError_t launch_build_twin(const int* tri, long long m, long long n, int* twin, int* cnt,
-                              int* start, int2* adj, long long* tile_sum, long long* tile_off,
-                              Counters* C, int sms, cudaStream_t s);
+// The twin array from tri (scratch: a table of twin_words(m) words).
+constexpr long long twin_words(long long m) { return 4 * m + 8 - 4 * m % 8; }
+cudaError_t launch_build_twin(const int* tri, long long m, long long n, int* twin, int* table,
+                              Counters* C, cudaStream_t s);
 // The twin array from a Neighbor array (convention 0: nb[3t+j] across the edge
 // opposite vertex j; 1: across the edge from vertex j to vertex j+1).
 cudaError_t launch_twin_from_neighbor(const int* tri, const int* nb, long long m, int convention,

@@ -3,189 +3,252 @@
 // runs from tri[h] to tri[3t + (k+1) % 3]; its twin is the half-edge running the
 // other way, or -1.
 //
-//   k_twin_count   outgoing half-edges per vertex (atomics), and the per-tile sums
-//                  of those counts for the tile scan;
-//   k_twin_start   each vertex's first slot: its tile's offset + an in-tile scan;
-//   k_twin_fill    every half-edge, with its destination, into its origin's slots;
-//   k_twin_match   h = u->v finds v->u among v's outgoing half-edges (about six
-//                  on a Delaunay mesh, one or two cache lines of (half-edge,
-//                  destination) pairs).  A directed edge used twice, or an edge
-//                  with more than two triangles, sets POLYLLA_ERR_TOPOLOGY: an
-//                  edge with more than two triangles repeats a directed edge,
-//                  and a repeated u->v is two hits for the thread of a v->u, or,
-//                  with no v->u, two entries in u's list.
+// One pass over tiles of kTwinTile triangles:
+//   in shared memory, each half-edge writes itself to its edge's slot and reads what
+//   stands there: of two twins one has lost the slot to the other and has found it.  Those
+//   that lost to another edge try a second slot;
+//   in a table of half-edges in memory, one word per edge, the half-edges left take a
+//   free word or find their twin in it, and for each pair of a tile its later half-edge
+//   takes a word, closed.  A third half-edge of an edge, or a second in the same
+//   direction, meets one of the others in a slot or a word: POLYLLA_ERR_TOPOLOGY.
 #include "polylla_internal.cuh"
 
 namespace polylla {
 
-constexpr int kTwinTile = kTriTile;  // vertices per tile of the count scan
+// What bounds it: the compare-and-swaps in L2 and their latency, one or two per edge, a
+// chain of about four for the longest of a warp, and the issue slots of the tiles' part.
+// Tiles: in an order with locality (a space-filling curve, a triangulator's insertion
+// order) 94 % of the half-edges have their twin among 512 triangles; those need neither a
+// second compare-and-swap nor the other's vertices from memory.  1,024 triangles: 96 %,
+// but fewer warps in flight; 256: 92 %.
+// Table: a word is a half-edge, whose vertices are looked up in tri, not a pair of
+// vertices.  An edge's words are near those of its region: 8 words, a sector, per vertex
+// (3 edges on average, those of which the vertex is the owner), then words anywhere,
+// then all in turn; the table is larger than the number of half-edges, so that a search
+// always ends.
+// Before: lists of half-edges per origin, searched for the twin (count, tile sums, scan,
+// first slots, fill, match).  With the launches and the wait, before and now: 4.0M
+// triangles of a mixture 227 us, 180; 400,000 of them 49, 31; 1,981 of a uniform mesh
+// 29, 20; 2.0M in random order (nothing to find in a tile) 222, 155; a fan of 100,000
+// (its hub's list) 5,540, 131.  The table alone, without tiles: 212, 36, 19, 107, 230.  A list
+// per owner with a warp matching 32 of them in shared memory: 204, 53, 35, 162.
+constexpr int kTwinTile = 512;  // triangles
+constexpr int kTwinEdges = 3 * kTwinTile;
+constexpr int kTwinPer = kTwinTile / kBlock;  // triangles of a thread
+constexpr unsigned kTwinSlots = 4096;         // of a tile: more than twice its edges
+constexpr unsigned kTwinGroup = 8;            // words of a vertex
+constexpr unsigned kTwinRandom = 64;          // words tried anywhere
+constexpr unsigned kTwinFree = 0xffffffffu;
+constexpr unsigned kTwinClosed = 0x80000000u;
 
-// Lanes of a warp holding the same vertex add to its count with one atomic (the
-// half-edges of neighbouring triangles share vertices).  The loop bound is
-// rounded up to whole warps so that every lane takes part in the match.
-__global__ void __launch_bounds__(kBlock) k_twin_count(const int* __restrict__ tri, long long m,
-                                                       long long n, int* __restrict__ cnt,
-                                                       Counters* C) {
-  const long long H = 3 * m;
-  const long long Hw = (H + 31) / 32 * 32;
+__device__ __forceinline__ unsigned twin_hash(unsigned a, unsigned b, unsigned i) {
+  unsigned x = a * 0x9e3779b1u ^ (b + i * 0x7f4a7c15u) * 0x85ebca6bu;
+  x ^= x >> 15;
+  x *= 0xc2b2ae35u;
+  return x ^ x >> 13;
+}
+
+// The i-th word tried for an edge of lo and hi, beyond its owner's group.
+__device__ __noinline__ unsigned twin_far(unsigned lo, unsigned hi, unsigned i, unsigned words) {
+  i -= kTwinGroup;
+  const unsigned r =
+      (unsigned)((unsigned long long)twin_hash(lo, hi, min(i, kTwinRandom)) * words >> 32);
+  return i <= kTwinRandom ? r : (unsigned)(((unsigned long long)r + (i - kTwinRandom)) % words);
+}
+
+// The i-th word tried for the edge of u and v; scale: groups per vertex, 32.32.
+__device__ __forceinline__ unsigned twin_word(int u, int v, unsigned i, unsigned words,
+                                              unsigned long long scale) {
+  // the owner: either vertex, so that a hub or a low id owns half of its edges
+  const unsigned lo = min(u, v), hi = max(u, v);
+  const bool low = (lo ^ hi) & 1;
+  if (i >= kTwinGroup) return twin_far(lo, hi, i, words);
+  return (unsigned)((low ? lo : hi) * scale >> 32) * kTwinGroup + ((low ? hi : lo) + i) % kTwinGroup;
+}
+
+// A vertex out of range is reported whatever else is wrong with the mesh.
+__device__ __forceinline__ void set_range_error(Counters* C) {
+  const int was = atomicCAS(&C->error, 0, (int)POLYLLA_ERR_RANGE);
+  if (was == (int)POLYLLA_ERR_TOPOLOGY) atomicCAS(&C->error, was, (int)POLYLLA_ERR_RANGE);
+  if (was == 0 || was == (int)POLYLLA_ERR_TOPOLOGY) C->err_info = 140;
+}
+
+// A slot of the tile's table for an edge: round r = 0, 1.
+__device__ __forceinline__ unsigned tile_slot(int u, int v, int r) {
+  const unsigned lo = min(u, v), hi = max(u, v);
+  const unsigned x = r ? lo * 0x85ebca6bu + hi * 0xc2b2ae35u : lo * 0x9e3779b1u + hi * 0x7feb352du;
+  return x / (unsigned)(0x100000000ull / kTwinSlots);
+}
+
+// Half-edge l = u -> v of a tile: its twin, when the edge's slot holds it (a half-edge
+// and the next of its triangle, 16 bits each).
+__device__ __forceinline__ void match_in_tile(const int* s_v, int* s_mate, int l, int u, int v,
+                                              unsigned slot, Counters* C) {
+  const int o = (int)(slot & 0xffff);
+  if (o == l) return;
+  const int a = s_v[o], b = s_v[slot >> 16];
+  if (a == v && b == u && u != v) {
+    s_mate[l] = o;
+    if (atomicExch(s_mate + o, l) != -1) set_error(C, POLYLLA_ERR_TOPOLOGY, 141);
+  } else if (a == u && b == v) {
+    set_error(C, POLYLLA_ERR_TOPOLOGY, 141);
+  }
+}
+
+// (6 blocks an SM, 40 registers: 180 us at 4.0M triangles; 4 blocks, nothing spilled: 208)
+__global__ void __launch_bounds__(kBlock, 6) k_twin_build(const int* __restrict__ tri, long long m,
+                                                          long long n, int* __restrict__ twin,
+                                                          unsigned* __restrict__ table,
+                                                          unsigned words, unsigned long long scale,
+                                                          Counters* C) {
+  __shared__ int s_v[kTwinEdges];
+  __shared__ int s_mate[kTwinEdges];
+  __shared__ unsigned s_slot[kTwinSlots];
+  __shared__ unsigned short s_list[kTwinEdges];
+  __shared__ int s_open;
   const int lane = threadIdx.x & 31;
-  for (long long h = blockIdx.x * (long long)blockDim.x + threadIdx.x; h < Hw;
-       h += (long long)gridDim.x * blockDim.x) {
-    int v = h < H ? __ldg(tri + h) : -1;
-    if (h < H && (v < 0 || v >= n)) {
-      set_error(C, POLYLLA_ERR_RANGE, 140);
-      v = -1;
-    }
-    const unsigned same = __match_any_sync(0xffffffffu, v);
-    if (v >= 0 && lane == __ffs(same) - 1) atomicAdd(cnt + v, __popc(same));
-  }
-}
-
-__global__ void __launch_bounds__(kBlock) k_twin_tiles(const int* __restrict__ cnt, long long n,
-                                                       long long* __restrict__ tile_sum) {
-  __shared__ long long sh[kBlock / 32];
-  const long long ntiles = (n + kTwinTile - 1) / kTwinTile;
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    long long s = 0;
-    for (int j = threadIdx.x; j < kTwinTile; j += kBlock) {
-      const long long v = tile * kTwinTile + j;
-      if (v < n) s += cnt[v];
-    }
-    const long long tot = block_sum(s, sh);
-    if (threadIdx.x == 0) {
-      tile_sum[2 * tile] = tot;
-      tile_sum[2 * tile + 1] = 0;
-    }
-  }
-}
-
-// start[v] = first slot of v; start[n] = 3m.  cnt is cleared for the fill.
-__global__ void __launch_bounds__(kBlock) k_twin_start(int* __restrict__ cnt, long long n,
-                                                       const long long* __restrict__ tile_off,
-                                                       int* __restrict__ start, long long m) {
-  __shared__ long long sh[kBlock / 32];
-  constexpr int kPer = kTwinTile / kBlock;
-  const long long ntiles = (n + kTwinTile - 1) / kTwinTile;
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const long long v0 = tile * kTwinTile + (long long)threadIdx.x * kPer;
-    int c[kPer];
-    long long s = 0;
+  for (long long t0 = (long long)blockIdx.x * kTwinTile; t0 < m;
+       t0 += (long long)gridDim.x * kTwinTile) {
+    const int base = (int)(3 * t0), count = (int)min((long long)kTwinEdges, 3 * (m - t0));
+    int v[kTwinPer][3];
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      c[j] = (v0 + j < n) ? cnt[v0 + j] : 0;
-      s += c[j];
-    }
-    long long tot;
-    long long p = tile_off[2 * tile] + block_exclusive_scan(s, &tot, sh);
+    for (int j = 0; j < kTwinPer; ++j) {
+      const int l = 3 * (threadIdx.x + j * kBlock);
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      if (v0 + j < n) {
-        start[v0 + j] = (int)p;
-        cnt[v0 + j] = 0;
+      for (int k = 0; k < 3; ++k) v[j][k] = l < count ? __ldg(tri + base + l + k) : -1;
+    }
+    if (threadIdx.x == 0) s_open = 0;
+#pragma unroll
+    for (int j = 0; j < kTwinPer; ++j) {
+      const int l = 3 * (threadIdx.x + j * kBlock);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (l < count && (v[j][k] < 0 || v[j][k] >= n)) {
+          set_range_error(C);
+          v[j][k] = -1;
+        }
+        s_v[l + k] = v[j][k];
+        s_mate[l + k] = -1;
       }
-      p += c[j];
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (min(v[j][k], v[j][(k + 1) % 3]) >= 0)
+          s_slot[tile_slot(v[j][k], v[j][(k + 1) % 3], 0)] = (l + k) | (l + (k + 1) % 3) << 16;
     }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) start[n] = (int)(3 * m);
-}
-
-// Each origin's slots: the half-edges' destinations in adj_dst, the half-edges
-// themselves at the same positions in adj_he.  Lanes with the same origin take
-// consecutive slots from one atomic.
-__global__ void __launch_bounds__(kBlock) k_twin_fill(const int* __restrict__ tri, long long m,
-                                                      long long n, const int* __restrict__ start,
-                                                      int* __restrict__ cnt,
-                                                      int* __restrict__ adj_dst,
-                                                      int* __restrict__ adj_he) {
-  const long long H = 3 * m;
-  const long long Hw = (H + 31) / 32 * 32;
-  const int lane = threadIdx.x & 31;
-  for (long long h = blockIdx.x * (long long)blockDim.x + threadIdx.x; h < Hw;
-       h += (long long)gridDim.x * blockDim.x) {
-    int v = h < H ? __ldg(tri + h) : -1;
-    if (v >= n) v = -1;
-    const unsigned same = __match_any_sync(0xffffffffu, v);
-    const int leader = __ffs(same) - 1;
-    int base = 0;
-    if (v >= 0 && lane == leader) base = atomicAdd(cnt + v, __popc(same));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (v < 0) continue;
-    const int q = start[v] + base + __popc(same & ((1u << lane) - 1u));
-    adj_dst[q] = __ldg(tri + he_next((int)h));
-    adj_he[q] = (int)h;
-  }
-}
-
-__global__ void __launch_bounds__(kBlock) k_twin_match(const int* __restrict__ tri, long long m,
-                                                       long long n, const int* __restrict__ start,
-                                                       const int* __restrict__ adj_dst,
-                                                       const int* __restrict__ adj_he,
-                                                       int* __restrict__ twin, Counters* C) {
-  const long long H = 3 * m;
-  for (long long h = blockIdx.x * (long long)blockDim.x + threadIdx.x; h < H;
-       h += (long long)gridDim.x * blockDim.x) {
-    const int u = __ldg(tri + h);
-    const int v = __ldg(tri + he_next((int)h));
-    if (u < 0 || u >= n || v < 0 || v >= n) {
-      twin[h] = -1;
-      continue;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kTwinPer; ++j) {
+      const int l = 3 * (threadIdx.x + j * kBlock);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (min(v[j][k], v[j][(k + 1) % 3]) >= 0)
+          match_in_tile(s_v, s_mate, l + k, v[j][k], v[j][(k + 1) % 3],
+                        s_slot[tile_slot(v[j][k], v[j][(k + 1) % 3], 0)], C);
     }
-    // the twin: v -> u among v's outgoing half-edges.  A second v -> u is a
-    // non-manifold edge.  A second u -> v shows up as two hits in the scan of
-    // u's list made for a v -> u, when there is one; so u's own list is scanned
-    // only when h has no twin
-    int g = -1, hits = 0;
-    const int b0 = start[v], b1 = start[v + 1];
-    for (int q = b0; q < b1; ++q) {
-      if (__ldg(adj_dst + q) == u) {
-        g = q;
-        ++hits;
+    __syncthreads();
+    // the half-edges that lost their slot to another edge, and those without a twin here
+#pragma unroll
+    for (int j = 0; j < kTwinPer; ++j) {
+      const int l = 3 * (threadIdx.x + j * kBlock);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const bool open = min(v[j][k], v[j][(k + 1) % 3]) >= 0 && s_mate[l + k] < 0;
+        const unsigned who = __ballot_sync(0xffffffffu, open);
+        int at = 0;
+        if (lane == 0 && who) at = atomicAdd(&s_open, __popc(who));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (open) s_list[at + __popc(who & ((1u << lane) - 1))] = (unsigned short)(l + k);
       }
     }
-    if (hits) g = __ldg(adj_he + g);
-    int same = 1;
-    if (hits == 0) {
-      same = 0;
-      const int a0 = start[u], a1 = start[u + 1];
-      for (int q = a0; q < a1; ++q) same += __ldg(adj_dst + q) == v;
+    __syncthreads();
+    const int opens = s_open;
+    for (int j = threadIdx.x; j < opens; j += kBlock) {
+      const int l = s_list[j], ln = he_next(l);
+      s_slot[tile_slot(s_v[l], s_v[ln], 1)] = l | ln << 16;
     }
-    if (hits > 1 || same != 1) set_error(C, POLYLLA_ERR_TOPOLOGY, 141);
-    twin[h] = g;
+    __syncthreads();
+    for (int j = threadIdx.x; j < opens; j += kBlock) {
+      const int l = s_list[j], u = s_v[l], w = s_v[he_next(l)];
+      match_in_tile(s_v, s_mate, l, u, w, s_slot[tile_slot(u, w, 1)], C);
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < count; l += kBlock) {
+      const int mate = s_mate[l];
+      twin[base + l] = mate >= 0 ? base + mate : -1;
+    }
+    __threadfence();  // the words of twin before their half-edges can be found
+    __syncthreads();
+    // the half-edges left, and the later one of each pair, into the table
+    unsigned open = 0, closed = 0;
+#pragma unroll
+    for (int j = 0; j < kTwinPer; ++j) {
+      const int l = 3 * (threadIdx.x + j * kBlock);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int mate = s_mate[l + k];
+        if (min(v[j][k], v[j][(k + 1) % 3]) >= 0 && l + k > mate) open |= 1u << (3 * j + k);
+        if (mate >= 0) closed |= 1u << (3 * j + k);
+      }
+    }
+    for (unsigned i = 0; open; ++i) {
+      unsigned o[kTwinPer][3];
+#pragma unroll
+      for (int j = 0; j < kTwinPer; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const unsigned bit = 1u << (3 * j + k);
+          if (!(open & bit)) continue;
+          const unsigned h = base + 3 * (threadIdx.x + j * kBlock) + k;
+          o[j][k] = atomicCAS(table + twin_word(v[j][k], v[j][(k + 1) % 3], i, words, scale),
+                              kTwinFree, closed & bit ? h | kTwinClosed : h);
+        }
+#pragma unroll
+      for (int j = 0; j < kTwinPer; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const unsigned bit = 1u << (3 * j + k);
+          if (!(open & bit)) continue;
+          if (o[j][k] == kTwinFree) {
+            open &= ~bit;
+            continue;
+          }
+          const int g = (int)(o[j][k] & ~kTwinClosed), u = v[j][k], w = v[j][(k + 1) % 3];
+          const int a = __ldg(tri + g), b = __ldg(tri + he_next(g));
+          if (a == w && b == u && u != w && !(closed & bit) && !(o[j][k] & kTwinClosed)) {
+            const int h = base + 3 * (threadIdx.x + j * kBlock) + k;
+            if (atomicCAS(twin + g, -1, h) != -1) set_error(C, POLYLLA_ERR_TOPOLOGY, 141);
+            twin[h] = g;
+            open &= ~bit;
+          } else if ((a == u && b == w) || (a == w && b == u)) {
+            set_error(C, POLYLLA_ERR_TOPOLOGY, 141);
+            open &= ~bit;
+          }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kTwinPer; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)  // an edge from a vertex to itself
+        if (v[j][k] >= 0 && v[j][k] == v[j][(k + 1) % 3]) {
+          const int h = base + 3 * (threadIdx.x + j * kBlock) + k;
+          twin[h] = h;
+        }
+    __syncthreads();  // (the next tile's vertices)
   }
 }
 
-cudaError_t launch_build_twin(const int* tri, long long m, long long n, int* twin, int* cnt,
-                              int* start, int2* adj, long long* tile_sum, long long* tile_off,
-                              Counters* C, int sms, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)n, s);
+cudaError_t launch_build_twin(const int* tri, long long m, long long n, int* twin, int* table,
+                              Counters* C, cudaStream_t s) {
+  const long long tiles = (m + kTwinTile - 1) / kTwinTile;
+  const long long words = twin_words(m);
+  const unsigned long long scale =
+      ((unsigned long long)(words / kTwinGroup) << 32) / (unsigned long long)n;
+  cudaError_t e = cudaMemsetAsync(table, 0xff, sizeof(int) * (size_t)words, s);
   if (e != cudaSuccess) return e;
-  static std::atomic<int> c1{0}, c2{0}, c3{0}, c4{0}, c5{0};
-  const long long H = 3 * m;
-  const long long ntiles = (n + kTwinTile - 1) / kTwinTile;
-  int g = resident_grid(reinterpret_cast<const void*>(k_twin_count), kBlock, 0,
-                        (H + kBlock - 1) / kBlock, &c1);
-  k_twin_count<<<g, kBlock, 0, s>>>(tri, m, n, cnt, C);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  g = resident_grid(reinterpret_cast<const void*>(k_twin_tiles), kBlock, 0, ntiles, &c2);
-  k_twin_tiles<<<g, kBlock, 0, s>>>(cnt, n, tile_sum);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_scan_tiles(tile_sum, tile_off, n, nullptr, n, kTwinTile, &C->scratch0,
-                             &C->scratch1, nullptr, 0, 0, C, s)) != cudaSuccess)
-    return e;
-  g = resident_grid(reinterpret_cast<const void*>(k_twin_start), kBlock, 0, ntiles, &c3);
-  k_twin_start<<<g, kBlock, 0, s>>>(cnt, n, tile_off, start, m);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // the pair buffer (3m int2) as two int arrays of 3m
-  int* adj_dst = reinterpret_cast<int*>(adj);
-  int* adj_he = adj_dst + H;
-  g = resident_grid(reinterpret_cast<const void*>(k_twin_fill), kBlock, 0,
-                    (H + kBlock - 1) / kBlock, &c4);
-  k_twin_fill<<<g, kBlock, 0, s>>>(tri, m, n, start, cnt, adj_dst, adj_he);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  g = resident_grid(reinterpret_cast<const void*>(k_twin_match), kBlock, 0,
-                    (H + kBlock - 1) / kBlock, &c5);
-  (void)sms;
-  k_twin_match<<<g, kBlock, 0, s>>>(tri, m, n, start, adj_dst, adj_he, twin, C);
+  static std::atomic<int> cap{0};
+  const int g = resident_grid(reinterpret_cast<const void*>(k_twin_build), kBlock, 0, tiles, &cap);
+  k_twin_build<<<g, kBlock, 0, s>>>(tri, m, n, twin, reinterpret_cast<unsigned*>(table),
+                                    (unsigned)words, scale, C);
   return cudaGetLastError();
 }
 
