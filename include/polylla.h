@@ -96,7 +96,8 @@ typedef struct {
   int64_t n_poly;         /* polygons after reparation */
   int64_t n_vtx;          /* their total length */
   /* Which device path handled the polygons of the last traversal / reparation
-   * pass (every path gives the same polygons; these show which ones ran): */
+   * pass (every path gives the same polygons; these show which ones ran; a polygon
+   * that a block took beside the walk counts as what the walk would have made it): */
   int64_t n_long;         /* polygons longer than the thread walk's cap (and, on
                              meshes of fewer than 2^16 triangles, polygons with three
                              or more tips), walked and split by one thread block each */

@@ -49,6 +49,7 @@ struct polylla_mesh {
 
   uint8_t* lab = nullptr;
   int* seeds = nullptr;
+  unsigned* len = nullptr;  // longest edge of each kLenChunk triangles (len_key)
   int* entry = nullptr;   // per seed: terminal half-edge, where its walk enters
   int* lepp_region = nullptr;  // per triangle: seed of its longest-edge path's end
   int* lepp_depth = nullptr;   // per triangle: links of that path
@@ -77,11 +78,13 @@ struct polylla_mesh {
   // the three kernels after the walk touch disjoint polygons: fork to two side
   // streams and join back (sequential in timing mode, for per-kernel times)
   cudaStream_t side[2] = {nullptr, nullptr};
+  cudaEvent_t walked = nullptr;
   cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
 
   // schedule: the walk's thread-per-seed cap and the long-polygon mode
   int walk_cap = kWalkCap;
   bool overlap = true;  // the kernels after the walk on side streams
+  bool beside = true;   // blocks beside the walk for the regions likely to be long
   bool rare_paths = false;  // polylla_debug_rare_paths
   int long_mode = 0;
   // polylla_run meshes a mesh of at most this many triangles in one thread block
@@ -182,7 +185,7 @@ void free_all(polylla_mesh* h) {
                   h->off_trav,  h->vtx_trav,   h->off_final,
                   h->seed_status, h->out_status,
                   h->vtx_final, h->C,         h->Dl.poly,   h->P.tip_h,
-                  h->Dm.poly,   h->entry,     h->Lg2.poly,
+                  h->Dm.poly,   h->entry,     h->Lg2.poly, h->len,
                   h->lepp_region, h->lepp_depth, h->trivertex};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -204,6 +207,7 @@ void free_all(polylla_mesh* h) {
     if (h->join[k]) cudaEventDestroy(h->join[k]);
   }
   if (h->fork) cudaEventDestroy(h->fork);
+  if (h->walked) cudaEventDestroy(h->walked);
 }
 
 // Device bytes of a handle's derived buffers for n vertices and m triangles (as
@@ -219,7 +223,8 @@ polylla_status alloc_derived(polylla_mesh* h) {
         cudaEventCreateWithFlags(&h->join[k], cudaEventDisableTiming) != cudaSuccess)
       return POLYLLA_ERR_CUDA;
   }
-  if (cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess)
+  if (cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->walked, cudaEventDisableTiming) != cudaSuccess)
     return POLYLLA_ERR_CUDA;
   const long long ntiles_tri = (m + kTriTile - 1) / kTriTile;
   const long long ntiles_poly = (m + kPolyTile - 1) / kPolyTile;
@@ -237,6 +242,7 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->lab, m + 4);
   ALLOC(h->seeds, m);
   ALLOC(h->entry, m);
+  ALLOC(h->len, m / kLenChunk + 1);
   ALLOC(h->lepp_region, m);
   ALLOC(h->lepp_depth, m);
   ALLOC(h->trivertex, n);
@@ -299,6 +305,7 @@ long long derived_bytes(long long n, long long m) {
   COUNT(c.lab, m + 4);
   COUNT(c.seeds, m);
   COUNT(c.entry, m);
+  COUNT(c.len, m / kLenChunk + 1);
   COUNT(c.tf, 3 * m);
   COUNT(c.loc, 3 * m);
   COUNT(c.vstamp, n);
@@ -366,7 +373,7 @@ polylla_status do_label(polylla_mesh* h, cudaStream_t s) {
   ++h->epoch;
   POLY_TRY(cuda_status(cudaMemsetAsync(h->C, 0, sizeof(Counters), s)));
   const int g1 = grid_for(h, (M.m + 3) / 4, kBlock);
-  POLY_TRY(launch(h, "label_max", s, [&] { return launch_label_max(M, h->lab, h->C, g1, s); }));
+  POLY_TRY(launch(h, "label_max", s, [&] { return launch_label_max(M, h->lab, h->beside ? h->len : nullptr, h->C, g1, s); }));
   const int g2 = grid_for(h, M.m, kTriTile);
   POLY_TRY(launch(h, "label_class", s, [&] {
     return launch_label_class(M, h->lab, h->tf, h->C, g2, s, !h->timing);
@@ -382,7 +389,9 @@ polylla_status do_seeds(polylla_mesh* h, cudaStream_t s) {
   const DevMesh& M = h->M;
   const int g = grid_for(h, M.m, 16 * kTriTile);
   POLY_TRY(launch(h, "seed_write", s, [&] {
-    return launch_seed_write(h->lab, M.m, h->seed_status, h->seeds, h->entry, h->C, g, s,
+    return launch_seed_write(h->lab, M.m, h->seed_status, h->seeds, h->entry,
+                             M, h->len,
+                             h->beside && M.m >= 2 * kEarlyMost ? h->Lg2.poly : nullptr, h->C, g, s,
                              !h->timing && h->phase == kLabeled);
   }));
   h->phase = kSeeded;
@@ -405,20 +414,40 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
     const size_t last = offsetof(Counters, seed_ticket);
     POLY_TRY(cuda_status(cudaMemsetAsync(reinterpret_cast<char*>(h->C) + first, 0, last - first, s)));
   }
-  const int gw = grid_for(h, M.m, kWalkThreads / 2);
-  POLY_TRY(launch(h, "walk", s, [&] {
-    return launch_walk(M, h->tf, h->entry, h->P, h->pool, h->Lg, h->Dl, h->Dm, h->walk_cap,
-                       repair, M.m < kSmallMeshTri ? kRsMaxSplit + 1 : 0, h->C, gw, s, pdl);
-  }));
-  // repair_one (this stream), repair_multi and long (side streams) at once
+  // blocks beside the walk for the regions that may be long: the stream's next kernel, so
+  // that they are placed first; the walk, a few us later, on a side stream
   const bool fork = !h->timing && h->overlap;
-  cudaStream_t s1 = s, s2 = s;
+  const bool beside = h->beside && !h->rare_paths && M.m >= 2 * kEarlyMost;
+  cudaStream_t s0 = s, s1 = s, s2 = s;  // walk and repair_one, long, repair_multi
   if (fork) {
-    POLY_TRY(cuda_status(cudaEventRecord(h->fork, s)));
-    for (int k = 0; k < 2; ++k)
-      POLY_TRY(cuda_status(cudaStreamWaitEvent(h->side[k], h->fork, 0)));
     s1 = h->side[0];
     s2 = h->side[1];
+  }
+  if (beside) {
+    if (fork) {
+      POLY_TRY(cuda_status(cudaEventRecord(h->fork, s)));
+      s0 = h->side[0];
+      s1 = s;
+      POLY_TRY(cuda_status(cudaStreamWaitEvent(s0, h->fork, 0)));
+    }
+    POLY_TRY(launch(h, "long_early", s1, [&] {
+      const LongList early{h->Lg2.poly, h->Lg2.cap};
+      return launch_long_early(M, h->lab, h->tf, h->seeds, h->P, h->F, h->pool, early, h->Lg,
+                               h->loc, h->vstamp, 2 * h->epoch + repair, repair, h->walk_cap, h->C,
+                               s1, pdl);
+    }));
+  }
+  const int gw = grid_for(h, M.m, kWalkThreads / 2);
+  POLY_TRY(launch(h, "walk", s0, [&] {
+    return launch_walk(M, h->tf, h->entry, h->P, h->pool, h->Lg, h->Dl, h->Dm, h->walk_cap,
+                       repair, M.m < kSmallMeshTri ? kRsMaxSplit + 1 : 0, beside, h->C, gw, s0,
+                       pdl && !beside);
+  }));
+  // repair_one (the walk's stream), repair_multi and long (others) at once
+  if (fork) {
+    POLY_TRY(cuda_status(cudaEventRecord(h->walked, s0)));
+    POLY_TRY(cuda_status(cudaStreamWaitEvent(s1, h->walked, 0)));
+    POLY_TRY(cuda_status(cudaStreamWaitEvent(s2, h->walked, 0)));
   }
   POLY_TRY(launch(h, "long", s1, [&] {
     return launch_long(M, h->lab, h->tf, h->seeds, h->P, h->F, h->pool, h->Lg, h->Lg2,
@@ -431,9 +460,9 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
                                  h->rare_paths, h->C,
                                  h->sms, s2);
     }));
-    POLY_TRY(launch(h, "repair_one", s, [&] {
+    POLY_TRY(launch(h, "repair_one", s0, [&] {
       return launch_repair_one(M, h->lab, h->tf, h->P, h->F, h->pool, h->Dl,
-                               h->rare_paths, h->C, h->sms, s, !h->timing);
+                               h->rare_paths, h->C, h->sms, s0, !h->timing);
     }));
   }
   if (fork) {
@@ -957,7 +986,7 @@ polylla_status polylla_get_stats(polylla_mesh_t h, polylla_stats* out) {
     out->n_tips = c.n_tips;
   }
   if (h->phase >= kTraversed || h->latest_csr == 1) {
-    out->n_long = c.n_long;
+    out->n_long = c.n_long + c.n_long_early;
     out->n_long_handoff = c.n_long2;
     out->n_long_seq = c.n_long_seq;
   }
@@ -965,8 +994,8 @@ polylla_status polylla_get_stats(polylla_mesh_t h, polylla_stats* out) {
     out->n_splits = c.n_splits;
     out->n_poly = c.n_poly;
     out->n_vtx = c.n_vtx;
-    out->n_one_tip = c.n_defer;
-    out->n_multi_tip = c.n_multi;
+    out->n_one_tip = c.n_defer + c.n_one_early;
+    out->n_multi_tip = c.n_multi + c.n_multi_early;
     out->n_multi_seq = c.n_multi_seq;
     out->n_one_chase = c.n_one_chase;
     out->n_multi_turn = c.n_multi_turn;
@@ -1161,6 +1190,7 @@ polylla_status polylla_batch_create(const int64_t* d_xy, const int64_t* d_vtx_of
     return POLYLLA_ERR_OOM;
   }
   b->mesh = h;
+  h->beside = false;  // thousands of meshes' border seeds: the walk has them
   cudaError_t e = dalloc(&b->tri_g, 3 * m);
   if (e == cudaSuccess) e = dalloc(&b->twin_g, 3 * m);
   if (e == cudaSuccess) e = dalloc(&b->d_tri_off, n_meshes + 1);

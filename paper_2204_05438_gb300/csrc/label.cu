@@ -89,17 +89,23 @@ __device__ __forceinline__ long long sqdist(longlong2 p, longlong2 q) {
 // ------------------------------------------------------------------ LabelMax
 // Longest edge by (exact squared length, then lower undirected id min(h, twin(h))).
 // The twin array is read only for triangles whose longest length is tied.
-__global__ void __launch_bounds__(kBlock, 6) k_label_max(DevMesh M, uint8_t* __restrict__ lab,
-                                                      Counters* C) {
+// With len, also the longest edge of each kLenChunk triangles, and of all of them in
+// C->max_len: what k_seed_write finds the long terminal edges by.
+// (5 blocks an SM: the length costs 2 registers over the 42 of 6 blocks, which then spill;
+// 2M triangles in random order 31.0 us, 27.5; 20M in order 105 either way, 96 without len)
+__global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __restrict__ lab,
+                                                         unsigned* __restrict__ len, Counters* C) {
   pdl_launch_dependents();
   const long long m = M.m, n = M.n;
   const long long ngroups = (m + 3) / 4;
+  unsigned seen = 0;  // the longest edge of this warp's triangles so far
   const longlong2* __restrict__ xy2 = reinterpret_cast<const longlong2*>(M.xy);
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < ngroups;
        g += (long long)gridDim.x * blockDim.x) {
     int v[12];
     load_tri_group(M.tri, g, m, v);
     unsigned packed = 0;
+    unsigned longest = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const long long t = 4 * g + j;
@@ -113,6 +119,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_label_max(DevMesh M, uint8_t* __r
       const longlong2 pa = __ldg(xy2 + a), pb = __ldg(xy2 + b), pc = __ldg(xy2 + c);
       const long long l0 = sqdist(pa, pb), l1 = sqdist(pb, pc), l2 = sqdist(pc, pa);
       const long long lmax = max(l0, max(l1, l2));
+      longest = max(longest, len_key(lmax));
       const int cnt = (l0 == lmax) + (l1 == lmax) + (l2 == lmax);
       int k;
       if (cnt == 1) {
@@ -142,14 +149,33 @@ __global__ void __launch_bounds__(kBlock, 6) k_label_max(DevMesh M, uint8_t* __r
     } else {
       for (int j = 0; t0 + j < m; ++j) lab[t0 + j] = (uint8_t)(packed >> (8 * j));
     }
+    if (len) {  // the longest edge of the warp's kLenChunk triangles, and of all
+      const long long lanes = ngroups - (g - g % 32);
+      const unsigned here =
+          __reduce_max_sync(lanes < 32 ? (1u << lanes) - 1u : 0xffffffffu, longest);
+      if (g % 32 == 0) {
+        len[g / 32] = here;
+        seen = max(seen, here);
+      }
+    }
+  }
+  if (len) {  // one atomic per block: one per warp took 6 us at 2M triangles in random order
+    __shared__ unsigned s_seen[kBlock / 32];
+    if (threadIdx.x % 32 == 0) s_seen[threadIdx.x / 32] = seen;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int w = 1; w < kBlock / 32; ++w) seen = max(seen, s_seen[w]);
+      atomicMax(&C->max_len, seen);
+    }
   }
 }
 
-cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, Counters* C, int grid,
+cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, unsigned* len, Counters* C, int grid,
                              cudaStream_t s) {
   static std::atomic<int> cap{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_label_max), kBlock, 0, grid, &cap);
-  k_label_max<<<grid, kBlock, 0, s>>>(M, lab, C);
+  k_label_max<<<grid, kBlock, 0, s>>>(M, lab, len, C);
   return cudaGetLastError();
 }
 
@@ -257,15 +283,31 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // With `entry` non-null, also the terminal half-edge 3t + k of each seed t (label
 // bits 0-1), where the walk enters its region.  The frontier half-edges (label bits
 // 2-4) are counted in C->n_front.
+// With `early`, the seeds whose regions may be long are listed (their entries carry
+// kEarlyBit): those whose terminal edge is a border edge (the label's frontier bit of
+// the longest edge; the slivers along a hull), and those whose terminal edge is at least a
+// 16th of the mesh's longest edge (the gaps between clusters).  On uniform and mixture
+// meshes of 1,000 to 1M points, 17-38 seeds of the first kind and 40-60 of the second
+// include every region of more than kWalkCap boundary edges.  A kind with more than
+// kEarlyMost seeds (a domain with holes; a mesh of edges all alike) says nothing, and
+// its seeds are the walk's like all others.
 constexpr int kSeedPer = 16;
 constexpr int kSeedSpan = kBlock * kSeedPer;   // triangles per sub-tile
 constexpr int kSeedSub = 4;                    // sub-tiles per look-back tile
 constexpr int kSeedTile = kSeedSub * kSeedSpan;
 
+__device__ __forceinline__ void list_early(int* early, int kind, long long i, Counters* C) {
+  const long long at =
+      (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_early[kind]), 1ull);
+  if (at < kEarlyMost) early[kind * kEarlyMost + at] = (int)i;
+}
+
 __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict__ lab, long long m,
                                                        unsigned long long* status,
                                                        int* __restrict__ seeds,
-                                                       int* __restrict__ entry, Counters* C) {
+                                                       int* __restrict__ entry,
+                                                       DevMesh M, const unsigned* __restrict__ len,
+                                                       int* __restrict__ early, Counters* C) {
   __shared__ int sw[kSeedSub][kBlock / 32];
   __shared__ int s_seed[kSeedSpan], s_entry[kSeedSpan];
   __shared__ long long s_tile, s_base;
@@ -275,6 +317,8 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long nbt = (m + kSeedTile - 1) / kSeedTile;
   const bool aligned16 = (reinterpret_cast<uintptr_t>(lab) & 15u) == 0;
+  const unsigned longest = early ? C->max_len : 0;
+  const unsigned far = longest > kLenFar ? longest - kLenFar : 0;
   for (;;) {
     if (threadIdx.x == 0)
       s_tile = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&C->seed_ticket), 1ull);
@@ -284,11 +328,13 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
     // this thread's 16 label bytes of each sub-tile (every load issued first)
     unsigned w[kSeedSub][4];
     unsigned smask[kSeedSub];
+    unsigned near = 0;  // bit j: the chunk of the sub-tile's 16 triangles has a long edge
     int incl[kSeedSub], cnt[kSeedSub];
 #pragma unroll
     for (int j = 0; j < kSeedSub; ++j) {
       const long long t0 = ((bt * kSeedSub + j) * kBlock + threadIdx.x) * kSeedPer;
       w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0;
+      if (early && t0 < m) near |= (unsigned)(len[t0 / kLenChunk] >= far) << j;
       if (t0 + kSeedPer <= m && aligned16) {
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(lab) + (t0 / kSeedPer));
         w[j][0] = v.x;
@@ -361,14 +407,30 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
         sm &= sm - 1;
         const unsigned wq = i < 8 ? (i < 4 ? w[j][0] : w[j][1]) : (i < 12 ? w[j][2] : w[j][3]);
         const int t = (int)(t0 + i);
-        s_seed[pos] = t;
-        s_entry[pos] = 3 * t + (int)((wq >> (8 * (i & 3))) & 3u);
+        const unsigned byte = wq >> (8 * (i & 3)), k = byte & 3u;
+        const bool border = early && (byte >> (2 + k) & 1u);  // its terminal edge
+        s_seed[pos] = t | (near >> j & 1u ? (int)kEarlyBit : 0);
+        s_entry[pos] = (3 * t + (int)k) | (border ? (int)kEarlyBit : 0);
         ++pos;
       }
       __syncthreads();
       for (int k = threadIdx.x; k < sub_total[j]; k += kBlock) {
-        seeds[base + k] = s_seed[k];
-        if (entry) entry[base + k] = s_entry[k];
+        const int t = s_seed[k] & ~(int)kEarlyBit;
+        int e = s_entry[k];
+        seeds[base + k] = t;
+        if (e < 0) {
+          list_early(early, 0, base + k, C);
+        } else if (s_seed[k] < 0 && *const_cast<volatile long long*>(&C->n_early[1]) <= kEarlyMost) {
+          const int a = M.tri[e], b = M.tri[he_next(e)];
+          if ((unsigned)a < (unsigned long long)M.n && (unsigned)b < (unsigned long long)M.n) {
+            const longlong2* xy2 = reinterpret_cast<const longlong2*>(M.xy);
+            if (len_key(sqdist(__ldg(xy2 + a), __ldg(xy2 + b))) >= far) {
+              list_early(early, 1, base + k, C);
+              e |= (int)kEarlyBit;
+            }
+          }
+        }
+        if (entry) entry[base + k] = e;
       }
       base += sub_total[j];
       __syncthreads();
@@ -390,11 +452,12 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
 }
 
 cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
-                              int* seeds, int* entry, Counters* C, int grid, cudaStream_t s,
-                              bool pdl) {
+                              int* seeds, int* entry, const DevMesh& M, const unsigned* len,
+                              int* early, Counters* C, int grid, cudaStream_t s, bool pdl) {
   static std::atomic<int> cap{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_seed_write), kBlock, 0, grid, &cap);
-  return launch_chain(k_seed_write, grid, kBlock, 0, s, pdl, lab, m, status, seeds, entry, C);
+  return launch_chain(k_seed_write, grid, kBlock, 0, s, pdl, lab, m, status, seeds, entry, M,
+                      len, early, C);
 }
 
 long long seed_tiles(long long m) { return (m + kSeedTile - 1) / kSeedTile; }

@@ -30,6 +30,14 @@
 //
 // A region too large for the shared-memory budget is handled by one thread of the
 // block with the sequential code (long_fallback).
+//
+// What bounds it: one region's chain of dependent loads and barriers (BFS levels, turns,
+// jumping rounds), 40-80 us, with the rest of the GPU idle when it follows the walk.
+// So the seeds whose regions may be long (k_seed_write lists them) are taken by blocks
+// that run beside the walk, whatever their length, and after the walk only what is
+// left: regions that were not listed, or too large for such a block.  A run, us, with all
+// long regions after the walk and now: 1M uniform points 218 and 175, with shuffled
+// triangles 273 and 217, 200,000 mixture points 100 and 94, 10M 909 and 887.
 #include "walk.cuh"
 
 namespace polylla {
@@ -44,6 +52,14 @@ constexpr int kLT = 4096;  // BFS queue: triangles of one long region
 constexpr int kSmallThreads = 128;
 constexpr int kSmallLM = 512;
 constexpr int kSmallLT = 512;
+// Beside the walk: 90 KB of shared memory, which leaves room on the SM for two or three
+// of the walk's blocks.  512 threads: 1M uniform points 178 us the run, 182 with 256; but
+// 20,000 with holes, whose 183 listed regions then take a second round, 74 and 68.  1,024
+// members: the longest of the 1M points (1,682) has to wait for the large blocks, 232.
+constexpr int kEarlyThreads = 512;  // 256 on meshes below kEarlyMesh triangles
+constexpr long long kEarlyMesh = 1 << 18;
+constexpr int kEarlyLM = 2048;
+constexpr int kEarlyLT = 2048;
 constexpr int kWarpLM = 128;  // one warp per polygon: up to 128 members and triangles
 constexpr int kWarpLT = 128;
 
@@ -249,6 +265,18 @@ __device__ void long_fallback(const DevMesh& M, uint8_t* lab, int* tf, int t0, l
   atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_splits), (unsigned long long)(cnt - 1));
 }
 
+// A polygon taken beside the walk counts as what the walk would have listed it as.
+__device__ void count_early(int L, int nt, int cap, int repair, long long m, unsigned long long by,
+                            Counters* C) {
+  const bool many = repair && m < kSmallMeshTri && nt > kRsMaxSplit;
+  long long* c = nullptr;
+  if (L > cap || many) c = &C->n_long_early;
+  else if (repair && nt) c = nt == 1 ? &C->n_one_early : &C->n_multi_early;
+  if (c) atomicAdd(reinterpret_cast<unsigned long long*>(c), by);
+  if (c == &C->n_multi_early && nt > kRsMaxSplit)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_multi_seq), by);
+}
+
 // Lg / n: the polygons of this launch.  over (nullable): where a polygon too large
 // for this block size goes (with the counter n_over) instead of the sequential path.
 template <int THREADS, int LM, int LT>
@@ -258,7 +286,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
                                                   const long long* n_list, LongList over,
                                                   long long* n_over, int* __restrict__ loc,
                                                   int* __restrict__ vstamp, int epoch, int repair,
-                                                  Counters* C) {
+                                                  int early, Counters* C) {
+  pdl_wait();  // the lists
   constexpr int kLM = LM;
   constexpr int kLT = LT;
   extern __shared__ int smem[];
@@ -280,9 +309,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
   __shared__ long long s_base, s_fbase;
   const int H = (int)(3 * M.m);
   const long long limit = 3 * M.m + 3;
-  const long long nl = min(*n_list, Lg.cap);
+  // early: of either kind all, or none, which the walk then has
+  const long long ne = early && n_list[0] <= kEarlyMost ? n_list[0] : 0;
+  const long long nl =
+      early ? ne + (n_list[1] <= kEarlyMost ? n_list[1] : 0) : min(*n_list, Lg.cap);
   for (long long j = blockIdx.x; j < nl; j += gridDim.x) {
-    const long long i = Lg.poly[j];
+    const long long i = Lg.poly[early && j >= ne ? kEarlyMost + j - ne : j];
     const int t0 = seeds[i];
     if (t0 < 0 || t0 >= M.m) {  // (the same for the whole block)
       if (threadIdx.x == 0) set_error(C, POLYLLA_ERR_LIMIT, 115);
@@ -420,6 +452,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
       P.pcnt[i] = 0;
       P.flen[i] = 0;
       atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_vtx_trav), (unsigned long long)L);
+      if (early) count_early(L, nt, early, repair, M.m, 1ull, C);
       if (nt) {
         atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tips), (unsigned long long)nt);
         atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tip_polys), 1ull);
@@ -553,6 +586,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
         atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_vtx_trav), 0ull - (unsigned long long)L);
         atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tips), 0ull - (unsigned long long)nt);
         atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_tip_polys), ~0ull);
+        if (early) count_early(L, nt, early, repair, M.m, ~0ull, C);
         if (over.poly && !s_fail) {
           const long long q =
               (long long)atomicAdd(reinterpret_cast<unsigned long long*>(n_over), 1ull);
@@ -823,7 +857,8 @@ cudaError_t launch_long_t(const DevMesh& M, uint8_t* lab, int* tf, const int* se
                           const PolyArrays& P, const FinalPieces& F, const Pool& pool,
                           const LongList& Lg, const long long* n_list,
                           const LongList& over, long long* n_over, int* loc, int* vstamp,
-                          int epoch, int repair, Counters* C, int grid, cudaStream_t s) {
+                          int epoch, int repair, int early, Counters* C, int grid, cudaStream_t s,
+                          bool pdl) {
   const size_t smem = sizeof(int) * (size_t)long_smem_ints<LM, LT>();
   static std::atomic<bool> attr[kMaxDevices];
   const cudaError_t e =
@@ -832,10 +867,19 @@ cudaError_t launch_long_t(const DevMesh& M, uint8_t* lab, int* tf, const int* se
   static std::atomic<int> cap{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_long<THREADS, LM, LT>), THREADS, smem,
                        grid, &cap);
-  k_long<THREADS, LM, LT><<<grid, THREADS, smem, s>>>(M, lab, tf, seeds, P, F, pool, Lg,
-                                                      n_list, over, n_over, loc, vstamp, epoch,
-                                                      repair, C);
-  return cudaGetLastError();
+  return launch_chain(k_long<THREADS, LM, LT>, grid, THREADS, smem, s, pdl, M, lab, tf, seeds, P, F,
+                      pool, Lg, n_list, over, n_over, loc, vstamp, epoch, repair, early, C);
+}
+
+cudaError_t launch_long_early(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
+                              const PolyArrays& P, const FinalPieces& F, const Pool& pool,
+                              const LongList& early, const LongList& Lg, int* loc, int* vstamp,
+                              int epoch, int repair, int cap, Counters* C, cudaStream_t s,
+                              bool pdl) {
+  const auto launch = M.m < kEarlyMesh ? launch_long_t<kEarlyThreads / 2, kEarlyLM, kEarlyLT>
+                                       : launch_long_t<kEarlyThreads, kEarlyLM, kEarlyLT>;
+  return launch(M, lab, tf, seeds, P, F, pool, early, C->n_early, Lg, &C->n_long, loc, vstamp,
+                epoch, repair, cap, C, 2 * kEarlyMost, s, pdl);
 }
 
 cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
@@ -846,20 +890,21 @@ cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seed
   if (mode == 0)  // large blocks only
     return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, P, F, pool, Lg,
                                                  &C->n_long, none, nullptr, loc, vstamp, epoch,
-                                                 repair, C, sms, s);
+                                                 repair, 0, C, sms, s, false);
   // small blocks (mode 1) or one warp per polygon (mode 2) first; the regions
   // they cannot hold, in large blocks
   cudaError_t e =
       mode == 2 ? launch_long_t<32, kWarpLM, kWarpLT>(M, lab, tf, seeds, P, F, pool, Lg,
                                                       &C->n_long, Lg2, &C->n_long2, loc, vstamp,
-                                                      epoch, repair, C, 32 * sms, s)
+                                                      epoch, repair, 0, C, 32 * sms, s,
+                                                      false)
                 : launch_long_t<kSmallThreads, kSmallLM, kSmallLT>(
                       M, lab, tf, seeds, P, F, pool, Lg, &C->n_long, Lg2, &C->n_long2, loc,
-                      vstamp, epoch, repair, C, 16 * sms, s);
+                      vstamp, epoch, repair, 0, C, 16 * sms, s, false);
   if (e != cudaSuccess) return e;
   return launch_long_t<kLongThreads, kLM, kLT>(M, lab, tf, seeds, P, F, pool, Lg2,
                                                &C->n_long2, none, nullptr, loc, vstamp, epoch,
-                                               repair, C, sms, s);
+                                               repair, 0, C, sms, s, false);
 }
 
 }  // namespace polylla

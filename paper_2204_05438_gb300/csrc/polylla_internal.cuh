@@ -24,6 +24,9 @@ constexpr int kTriTile = kBlock * kTriPerThread;  // 1024 triangles per seed-cou
 constexpr long long kMaxTriangles = 1ll << 29;
 constexpr long long kMaxVertices = 1ll << 30;
 constexpr int kWalkThreads = 256;  // k_walk block
+constexpr int kEarlyMost = 256;    // seeds of either kind for blocks beside the walk, at most
+constexpr unsigned kEarlyBit = 0x80000000u;  // of their entries
+constexpr int kLenChunk = 128;               // triangles per word of the length array
 constexpr int kWalkCap = 64;       // longer polygons go to one thread block each (long.cu)
 constexpr int kPolyTile = kBlock;              // per-polygon scans: one polygon per thread
 
@@ -43,6 +46,9 @@ struct Counters {
   long long n_defer;      // polygons with one tip, left to k_repair_one
   long long n_multi;      // polygons with several tips, left to k_repair_multi
   long long ticket;       // tile tickets of the single-pass (look-back) scans
+  long long n_long_early; // of the polygons taken beside the walk: longer than the walk cap,
+  long long n_one_early;  // with one tip,
+  long long n_multi_early; // with several
   long long n_long2;      // long polygons handed from the small blocks to the large ones
   long long n_long_seq;   // long regions too large for a block, walked by one thread
   long long n_multi_seq;  // several-tip polygons with more tips than the node list holds
@@ -51,11 +57,19 @@ struct Counters {
   long long seed_ticket;  // tile tickets of the seed compaction's look-back
   long long seed_done;    // its completed look-backs (the last one clears the status)
   long long out_done;     // the output pass's completed look-backs (likewise)
+  long long n_early[2];   // seeds listed for the blocks beside the walk: with a border edge as
+                          // terminal edge, with a long one (k_seed_write)
+  unsigned max_len;       // len_key of the longest edge
   long long scratch0;     // split scratch of the one-block path
   long long n_block;      // polygons meshed by the one-block path (block.cu)
   int error;              // first device error (polylla_status), 0 if none
   int err_info;
 };
+
+// Squared lengths as 32 bits that keep their order (float, towards zero); that of an
+// edge 16 times shorter is kLenFar below.
+constexpr unsigned kLenFar = 8u << 23;
+__device__ __forceinline__ unsigned len_key(long long sq) { return __float_as_uint(__ll2float_rz(sq)); }
 
 struct DevMesh {
   const long long* xy;  // 2n
@@ -238,7 +252,7 @@ inline cudaError_t smem_limit_once(const void* kernel, int bytes, std::atomic<bo
 // ----------------------------------------------------------------- launchers
 // Every launcher enqueues one kernel on `s` and returns the launch error.
 cudaError_t launch_validate(const DevMesh& M, Counters* C, int grid, cudaStream_t s);
-cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, Counters* C, int grid,
+cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, unsigned* len, Counters* C, int grid,
                              cudaStream_t s);
 // pdl: launch with programmatic stream serialization (the previous operation on
 // the stream is a kernel)
@@ -248,8 +262,10 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // non-null), C->n_seeds and C->n_front in one pass:
 // look-back over `status` (seed_tiles(m) words, zero at the first use; left zero)
 // with tickets from C->seed_ticket (zero at the start).
+// len, early (nullable): see k_seed_write.
 cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
-                              int* seeds, int* entry, Counters* C, int grid, cudaStream_t s,
+                              int* seeds, int* entry, const DevMesh& M, const unsigned* len,
+                              int* early, Counters* C, int grid, cudaStream_t s,
                               bool pdl);
 long long seed_tiles(long long m);
 // Per polygon of the traversal (index = seed order), capacity m.
@@ -298,8 +314,8 @@ constexpr int kRsMaxSplit = 8;  // tips that a warp splits together (k_repair_mu
 constexpr long long kSmallMeshTri = 1ll << 16;  // meshes below this: more go to blocks
 cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,
                         const Pool& pool, const LongList& Lg, const LongList& D1,
-                        const LongList& Dm, int cap, int repair, int tips_to_long, Counters* C,
-                        int grid, cudaStream_t s, bool pdl);
+                        const LongList& Dm, int cap, int repair, int tips_to_long, int beside,
+                        Counters* C, int grid, cudaStream_t s, bool pdl);
 // One thread per polygon with one tip / one warp per polygon with several tips (listed
 // by k_walk).
 cudaError_t launch_repair_one(const DevMesh& M, uint8_t* lab, int* tf, const PolyArrays& P,
@@ -311,7 +327,12 @@ cudaError_t launch_repair_multi(const DevMesh& M, uint8_t* lab, int* tf, const P
 // One block per long polygon: gather, rank and, if `repair`, split.  mode 0:
 // large blocks only; mode 1: small blocks first, the regions they cannot hold
 // (listed in Lg2) then in large blocks; mode 2: the same with one-warp blocks
-// first.
+// first.  launch_long_early: the listed seeds' polygons, of any length, beside the walk.
+cudaError_t launch_long_early(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
+                              const PolyArrays& P, const FinalPieces& F, const Pool& pool,
+                              const LongList& early, const LongList& Lg, int* loc, int* vstamp,
+                              int epoch, int repair, int cap, Counters* C, cudaStream_t s,
+                              bool pdl);
 cudaError_t launch_long(const DevMesh& M, uint8_t* lab, int* tf, const int* seeds,
                         const PolyArrays& P, const FinalPieces& F, const Pool& pool,
                         const LongList& Lg, const LongList& Lg2, int* loc, int* vstamp, int epoch,

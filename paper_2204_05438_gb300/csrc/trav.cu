@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
                                                           PolyArrays P, Pool pool, LongList Lg,
                                                           LongList D1, LongList Dm, int cap,
                                                           int repair, int tips_to_long,
-                                                          Counters* C) {
+                                                          int beside, Counters* C) {
   extern __shared__ __align__(16) unsigned char walk_smem[];
   pdl_wait();  // the tf words, seeds and entries
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -137,6 +137,8 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
   const int* __restrict__ tri = M.tri;
   const int n = (int)C->n_seeds;  // below 2^29
   const int H = (int)(3 * M.m);
+  const bool early0 = beside && C->n_early[0] <= kEarlyMost,
+             early1 = beside && C->n_early[1] <= kEarlyMost;
   // polygons with 2 to this many tips leave their half-edges to the several-tip kernel
   const int most_rec = tips_to_long > 0 ? min(tips_to_long - 1, kRsMaxSplit) : kRsMaxSplit;
   unsigned st_len = 0, st_tips = 0, st_tippolys = 0;
@@ -150,12 +152,15 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
   int n1 = 0, nm = 0;  // entries of the warp's list buffers
   for (int base = ((int)blockIdx.x * kWalkWarps + warp) * per; base < n; base += warps * per) {
     const int i = base + lane;
-    int e0 = lane < per && i < n ? __ldg(entry + i) : -1;
+    const bool any = lane < per && i < n;
+    const int raw = any ? __ldg(entry + i) : 0;
+    int e0 = any ? raw & ~(int)kEarlyBit : -1;
     if (e0 >= H) {  // (no seed pass writes one)
       set_error(C, POLYLLA_ERR_LIMIT, 51);
       e0 = -1;
     }
     int x0 = e0 >= 0 ? __ldg(tf + e0) : -1;
+    if (raw < 0 && (x0 < 0 ? early0 : early1)) e0 = -1;  // a block has it
     bool big = false;  // too long for a walk: left to a thread block
     for (int b0 = 0; b0 < per && base + b0 < n;) {
       const bool taken = e0 >= 0 && lane >= b0 && lane < b0 + width;
@@ -490,8 +495,8 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
 
 cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,
                         const Pool& pool, const LongList& Lg, const LongList& D1,
-                        const LongList& Dm, int cap, int repair, int tips_to_long, Counters* C,
-                        int grid, cudaStream_t s, bool pdl) {
+                        const LongList& Dm, int cap, int repair, int tips_to_long, int beside,
+                        Counters* C, int grid, cudaStream_t s, bool pdl) {
   if (cap < 16 || cap > kWalkCap || cap % 16) return cudaErrorInvalidValue;
   constexpr size_t smem = sizeof(WalkBuf) * kWalkWarps;
   static std::atomic<bool> attr[kMaxDevices];
@@ -500,7 +505,7 @@ cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const
   static std::atomic<int> resident{0};
   grid = resident_grid(reinterpret_cast<const void*>(k_walk), kWalkThreads, smem, grid, &resident);
   return launch_chain(k_walk, grid, kWalkThreads, smem, s, pdl, M, tf, entry, P, pool, Lg, D1, Dm,
-                      cap, repair, tips_to_long, C);
+                      cap, repair, tips_to_long, beside, C);
 }
 
 __device__ __forceinline__ unsigned long long vkey(int origin, int h) {
