@@ -267,7 +267,7 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->F.len, h->F.cap);
   ALLOC(h->F.h, h->F.cap);
   ALLOC(h->pool.v, h->pool.cap);
-  ALLOC(h->seed_status, seed_tiles(m) + 1);
+  ALLOC(h->seed_status, seed_tiles(m, true) + 1);
   ALLOC(h->out_status, ntiles + 1);
   ALLOC(h->off_trav, m + 1);
   ALLOC(h->vtx_trav, 3 * m);
@@ -284,7 +284,7 @@ polylla_status alloc_derived(polylla_mesh* h) {
   if (e == cudaSuccess) e = cudaMemsetAsync(h->vstamp, 0, sizeof(int) * (size_t)n, s0);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(h->seed_status, 0,
-                        sizeof(unsigned long long) * (size_t)(seed_tiles(m) + 1), s0);
+                        sizeof(unsigned long long) * (size_t)(seed_tiles(m, true) + 1), s0);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(h->out_status, 0, sizeof(unsigned long long) * (size_t)(ntiles + 1), s0);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->C, 0, sizeof(Counters), s0);
@@ -329,7 +329,7 @@ long long derived_bytes(long long n, long long m) {
   COUNT(c.F.len, c.F.cap);
   COUNT(c.F.h, c.F.cap);
   COUNT(c.pool.v, c.pool.cap);
-  COUNT(c.seed_status, seed_tiles(m) + 1);
+  COUNT(c.seed_status, seed_tiles(m, true) + 1);
   COUNT(c.out_status, ntiles + 1);
   COUNT(c.off_trav, m + 1);
   COUNT(c.vtx_trav, 3 * m);
@@ -363,6 +363,11 @@ polylla_status check_handle(polylla_mesh* h) {
 }
 
 // ---------------------------------------------------------------- phases
+// Whether blocks beside the walk take the regions that may be long.
+bool beside(const polylla_mesh* h) {
+  return h->beside && !h->rare_paths && h->M.m >= 2 * kEarlyMost && h->M.m <= kBesideMost;
+}
+
 polylla_status do_label(polylla_mesh* h, cudaStream_t s) {
   const Range range("polylla label");
   const DevMesh& M = h->M;
@@ -373,7 +378,9 @@ polylla_status do_label(polylla_mesh* h, cudaStream_t s) {
   ++h->epoch;
   POLY_TRY(cuda_status(cudaMemsetAsync(h->C, 0, sizeof(Counters), s)));
   const int g1 = grid_for(h, (M.m + 3) / 4, kBlock);
-  POLY_TRY(launch(h, "label_max", s, [&] { return launch_label_max(M, h->lab, h->beside ? h->len : nullptr, h->C, g1, s); }));
+  POLY_TRY(launch(h, "label_max", s, [&] {
+    return launch_label_max(M, h->lab, beside(h) ? h->len : nullptr, h->C, g1, s);
+  }));
   const int g2 = grid_for(h, M.m, kTriTile);
   POLY_TRY(launch(h, "label_class", s, [&] {
     return launch_label_class(M, h->lab, h->tf, h->C, g2, s, !h->timing);
@@ -387,11 +394,9 @@ polylla_status do_label(polylla_mesh* h, cudaStream_t s) {
 polylla_status do_seeds(polylla_mesh* h, cudaStream_t s) {
   const Range range("polylla seeds");
   const DevMesh& M = h->M;
-  const int g = grid_for(h, M.m, 16 * kTriTile);
   POLY_TRY(launch(h, "seed_write", s, [&] {
-    return launch_seed_write(h->lab, M.m, h->seed_status, h->seeds, h->entry,
-                             M, h->len,
-                             h->beside && M.m >= 2 * kEarlyMost ? h->Lg2.poly : nullptr, h->C, g, s,
+    return launch_seed_write(h->lab, M.m, h->seed_status, h->seeds, h->entry, M, h->len,
+                             beside(h) ? h->Lg2.poly : nullptr, true, h->C, s,
                              !h->timing && h->phase == kLabeled);
   }));
   h->phase = kSeeded;
@@ -417,13 +422,13 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
   // blocks beside the walk for the regions that may be long: the stream's next kernel, so
   // that they are placed first; the walk, a few us later, on a side stream
   const bool fork = !h->timing && h->overlap;
-  const bool beside = h->beside && !h->rare_paths && M.m >= 2 * kEarlyMost;
+  const bool early = beside(h);
   cudaStream_t s0 = s, s1 = s, s2 = s;  // walk and repair_one, long, repair_multi
   if (fork) {
     s1 = h->side[0];
     s2 = h->side[1];
   }
-  if (beside) {
+  if (early) {
     if (fork) {
       POLY_TRY(cuda_status(cudaEventRecord(h->fork, s)));
       s0 = h->side[0];
@@ -431,8 +436,8 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
       POLY_TRY(cuda_status(cudaStreamWaitEvent(s0, h->fork, 0)));
     }
     POLY_TRY(launch(h, "long_early", s1, [&] {
-      const LongList early{h->Lg2.poly, h->Lg2.cap};
-      return launch_long_early(M, h->lab, h->tf, h->seeds, h->P, h->F, h->pool, early, h->Lg,
+      const LongList listed{h->Lg2.poly, h->Lg2.cap};
+      return launch_long_early(M, h->lab, h->tf, h->seeds, h->P, h->F, h->pool, listed, h->Lg,
                                h->loc, h->vstamp, 2 * h->epoch + repair, repair, h->walk_cap, h->C,
                                s1, pdl);
     }));
@@ -440,8 +445,8 @@ polylla_status do_polygons(polylla_mesh* h, cudaStream_t s, int repair, long lon
   const int gw = grid_for(h, M.m, kWalkThreads / 2);
   POLY_TRY(launch(h, "walk", s0, [&] {
     return launch_walk(M, h->tf, h->entry, h->P, h->pool, h->Lg, h->Dl, h->Dm, h->walk_cap,
-                       repair, M.m < kSmallMeshTri ? kRsMaxSplit + 1 : 0, beside, h->C, gw, s0,
-                       pdl && !beside);
+                       repair, M.m < kSmallMeshTri ? kRsMaxSplit + 1 : 0, early, h->C, gw, s0,
+                       pdl && !early);
   }));
   // repair_one (the walk's stream), repair_multi and long (others) at once
   if (fork) {

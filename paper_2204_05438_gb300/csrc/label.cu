@@ -91,9 +91,10 @@ __device__ __forceinline__ long long sqdist(longlong2 p, longlong2 q) {
 // The twin array is read only for triangles whose longest length is tied.
 // With len, also the longest edge of each kLenChunk triangles, and of all of them in
 // C->max_len: what k_seed_write finds the long terminal edges by.
-// (5 blocks an SM: the length costs 2 registers over the 42 of 6 blocks, which then spill;
-// 2M triangles in random order 31.0 us, 27.5; 20M in order 105 either way, 96 without len)
-__global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __restrict__ lab,
+// (5 blocks an SM then: with the 42 registers of 6 blocks it spills, 31.0 us against 27.5 at
+// 2M triangles in random order; 8M in order 49 us, 45 without len)
+template <bool LEN>
+__global__ void __launch_bounds__(kBlock, LEN ? 5 : 6) k_label_max(DevMesh M, uint8_t* __restrict__ lab,
                                                          unsigned* __restrict__ len, Counters* C) {
   pdl_launch_dependents();
   const long long m = M.m, n = M.n;
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __r
       const longlong2 pa = __ldg(xy2 + a), pb = __ldg(xy2 + b), pc = __ldg(xy2 + c);
       const long long l0 = sqdist(pa, pb), l1 = sqdist(pb, pc), l2 = sqdist(pc, pa);
       const long long lmax = max(l0, max(l1, l2));
-      longest = max(longest, len_key(lmax));
+      if (LEN) longest = max(longest, len_key(lmax));
       const int cnt = (l0 == lmax) + (l1 == lmax) + (l2 == lmax);
       int k;
       if (cnt == 1) {
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __r
     } else {
       for (int j = 0; t0 + j < m; ++j) lab[t0 + j] = (uint8_t)(packed >> (8 * j));
     }
-    if (len) {  // the longest edge of the warp's kLenChunk triangles, and of all
+    if (LEN) {  // the longest edge of the warp's kLenChunk triangles, and of all
       const long long lanes = ngroups - (g - g % 32);
       const unsigned here =
           __reduce_max_sync(lanes < 32 ? (1u << lanes) - 1u : 0xffffffffu, longest);
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __r
       }
     }
   }
-  if (len) {  // one atomic per block: one per warp took 6 us at 2M triangles in random order
+  if (LEN) {  // one atomic per block: one per warp took 6 us at 2M triangles in random order
     __shared__ unsigned s_seen[kBlock / 32];
     if (threadIdx.x % 32 == 0) s_seen[threadIdx.x / 32] = seen;
     __syncthreads();
@@ -171,12 +172,18 @@ __global__ void __launch_bounds__(kBlock, 5) k_label_max(DevMesh M, uint8_t* __r
   }
 }
 
+template <bool LEN>
+cudaError_t launch_label_max_t(const DevMesh& M, uint8_t* lab, unsigned* len, Counters* C, int grid,
+                               cudaStream_t s) {
+  static std::atomic<int> cap{0};
+  grid = resident_grid(reinterpret_cast<const void*>(k_label_max<LEN>), kBlock, 0, grid, &cap);
+  k_label_max<LEN><<<grid, kBlock, 0, s>>>(M, lab, len, C);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_label_max(const DevMesh& M, uint8_t* lab, unsigned* len, Counters* C, int grid,
                              cudaStream_t s) {
-  static std::atomic<int> cap{0};
-  grid = resident_grid(reinterpret_cast<const void*>(k_label_max), kBlock, 0, grid, &cap);
-  k_label_max<<<grid, kBlock, 0, s>>>(M, lab, len, C);
-  return cudaGetLastError();
+  return (len ? launch_label_max_t<true> : launch_label_max_t<false>)(M, lab, len, C, grid, s);
 }
 
 // ------------------------------------------------------------------ LabelSeed + LabelFrontier
@@ -293,8 +300,12 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // its seeds are the walk's like all others.
 constexpr int kSeedPer = 16;
 constexpr int kSeedSpan = kBlock * kSeedPer;   // triangles per sub-tile
-constexpr int kSeedSub = 4;                    // sub-tiles per look-back tile
-constexpr int kSeedTile = kSeedSub * kSeedSpan;
+// Sub-tiles per look-back tile: 4, or 1 on meshes of at most kSeedSmall triangles, where
+// 4 leave most of the GPU idle (us with 4 and 1, this kernel and the run: 29,667 triangles
+// with holes 22 and 12, 75 and 63; 400,000 of a mixture 16 and 12, 93 and 90; 1.4M 20 and
+// 15, 136 and 131; 2.0M uniform 21 and 19, 174 and 175).
+constexpr int kSeedSub = 4;
+constexpr long long kSeedSmall = 1 << 21;
 
 __device__ __forceinline__ void list_early(int* early, int kind, long long i, Counters* C) {
   const long long at =
@@ -302,12 +313,14 @@ __device__ __forceinline__ void list_early(int* early, int kind, long long i, Co
   if (at < kEarlyMost) early[kind * kEarlyMost + at] = (int)i;
 }
 
+template <int kSeedSub, bool EARLY>
 __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict__ lab, long long m,
                                                        unsigned long long* status,
                                                        int* __restrict__ seeds,
                                                        int* __restrict__ entry,
                                                        DevMesh M, const unsigned* __restrict__ len,
                                                        int* __restrict__ early, Counters* C) {
+  constexpr int kSeedTile = kSeedSub * kSeedSpan;
   __shared__ int sw[kSeedSub][kBlock / 32];
   __shared__ int s_seed[kSeedSpan], s_entry[kSeedSpan];
   __shared__ long long s_tile, s_base;
@@ -317,7 +330,7 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long nbt = (m + kSeedTile - 1) / kSeedTile;
   const bool aligned16 = (reinterpret_cast<uintptr_t>(lab) & 15u) == 0;
-  const unsigned longest = early ? C->max_len : 0;
+  const unsigned longest = EARLY ? C->max_len : 0;
   const unsigned far = longest > kLenFar ? longest - kLenFar : 0;
   for (;;) {
     if (threadIdx.x == 0)
@@ -334,7 +347,8 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
     for (int j = 0; j < kSeedSub; ++j) {
       const long long t0 = ((bt * kSeedSub + j) * kBlock + threadIdx.x) * kSeedPer;
       w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0;
-      if (early && t0 < m) near |= (unsigned)(len[t0 / kLenChunk] >= far) << j;
+      if constexpr (EARLY)
+        if (t0 < m) near |= (unsigned)(len[t0 / kLenChunk] >= far) << j;
       if (t0 + kSeedPer <= m && aligned16) {
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(lab) + (t0 / kSeedPer));
         w[j][0] = v.x;
@@ -408,7 +422,7 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
         const unsigned wq = i < 8 ? (i < 4 ? w[j][0] : w[j][1]) : (i < 12 ? w[j][2] : w[j][3]);
         const int t = (int)(t0 + i);
         const unsigned byte = wq >> (8 * (i & 3)), k = byte & 3u;
-        const bool border = early && (byte >> (2 + k) & 1u);  // its terminal edge
+        const bool border = EARLY && (byte >> (2 + k) & 1u);  // its terminal edge
         s_seed[pos] = t | (near >> j & 1u ? (int)kEarlyBit : 0);
         s_entry[pos] = (3 * t + (int)k) | (border ? (int)kEarlyBit : 0);
         ++pos;
@@ -418,15 +432,17 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
         const int t = s_seed[k] & ~(int)kEarlyBit;
         int e = s_entry[k];
         seeds[base + k] = t;
-        if (e < 0) {
-          list_early(early, 0, base + k, C);
-        } else if (s_seed[k] < 0 && *const_cast<volatile long long*>(&C->n_early[1]) <= kEarlyMost) {
-          const int a = M.tri[e], b = M.tri[he_next(e)];
-          if ((unsigned)a < (unsigned long long)M.n && (unsigned)b < (unsigned long long)M.n) {
-            const longlong2* xy2 = reinterpret_cast<const longlong2*>(M.xy);
-            if (len_key(sqdist(__ldg(xy2 + a), __ldg(xy2 + b))) >= far) {
-              list_early(early, 1, base + k, C);
-              e |= (int)kEarlyBit;
+        if constexpr (EARLY) {
+          if (e < 0) {
+            list_early(early, 0, base + k, C);
+          } else if (s_seed[k] < 0 && *const_cast<volatile long long*>(&C->n_early[1]) <= kEarlyMost) {
+            const int a = M.tri[e], b = M.tri[he_next(e)];
+            if ((unsigned)a < (unsigned long long)M.n && (unsigned)b < (unsigned long long)M.n) {
+              const longlong2* xy2 = reinterpret_cast<const longlong2*>(M.xy);
+              if (len_key(sqdist(__ldg(xy2 + a), __ldg(xy2 + b))) >= far) {
+                list_early(early, 1, base + k, C);
+                e |= (int)kEarlyBit;
+              }
             }
           }
         }
@@ -451,15 +467,31 @@ __global__ void __launch_bounds__(kBlock) k_seed_write(const uint8_t* __restrict
   }
 }
 
-cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
-                              int* seeds, int* entry, const DevMesh& M, const unsigned* len,
-                              int* early, Counters* C, int grid, cudaStream_t s, bool pdl) {
+template <int SUB, bool EARLY>
+cudaError_t launch_seed_write_t(const uint8_t* lab, long long m, unsigned long long* status,
+                                int* seeds, int* entry, const DevMesh& M, const unsigned* len,
+                                int* early, Counters* C, cudaStream_t s, bool pdl) {
   static std::atomic<int> cap{0};
-  grid = resident_grid(reinterpret_cast<const void*>(k_seed_write), kBlock, 0, grid, &cap);
-  return launch_chain(k_seed_write, grid, kBlock, 0, s, pdl, lab, m, status, seeds, entry, M,
+  const int grid = resident_grid(reinterpret_cast<const void*>(k_seed_write<SUB, EARLY>), kBlock, 0,
+                                 (m + SUB * kSeedSpan - 1) / (SUB * kSeedSpan), &cap);
+  return launch_chain(k_seed_write<SUB, EARLY>, grid, kBlock, 0, s, pdl, lab, m, status, seeds, entry, M,
                       len, early, C);
 }
 
-long long seed_tiles(long long m) { return (m + kSeedTile - 1) / kSeedTile; }
+cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
+                              int* seeds, int* entry, const DevMesh& M, const unsigned* len,
+                              int* early, bool small, Counters* C, cudaStream_t s, bool pdl) {
+  const bool one = small && m <= kSeedSmall;
+  const auto launch =
+      early ? (one ? launch_seed_write_t<1, true> : launch_seed_write_t<kSeedSub, true>)
+            : (one ? launch_seed_write_t<1, false> : launch_seed_write_t<kSeedSub, false>);
+  return launch(lab, m, status, seeds, entry, M, len, early, C, s, pdl);
+}
+
+long long seed_tiles(long long m, bool small) {
+  const long long large = (m + kSeedSub * kSeedSpan - 1) / (kSeedSub * kSeedSpan);
+  const long long n = small ? (std::min(m, kSeedSmall) + kSeedSpan - 1) / kSeedSpan : 0;
+  return std::max(large, n);
+}
 
 }  // namespace polylla

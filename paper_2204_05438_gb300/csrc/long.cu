@@ -37,7 +37,7 @@
 // that run beside the walk, whatever their length, and after the walk only what is
 // left: regions that were not listed, or too large for such a block.  A run, us, with all
 // long regions after the walk and now: 1M uniform points 218 and 175, with shuffled
-// triangles 273 and 217, 200,000 mixture points 100 and 94, 10M 909 and 887.
+// triangles 273 and 217, 2M uniform points 334 and 282, 200,000 mixture points 100 and 94.
 #include "walk.cuh"
 
 namespace polylla {
@@ -58,6 +58,9 @@ constexpr int kSmallLT = 512;
 // members: the longest of the 1M points (1,682) has to wait for the large blocks, 232.
 constexpr int kEarlyThreads = 512;  // 256 on meshes below kEarlyMesh triangles
 constexpr long long kEarlyMesh = 1 << 18;
+// Above this, large blocks: 2M uniform points have a region of more than 2,048 triangles, whose
+// time after the walk made the run 359 us instead of 282.
+constexpr long long kEarlyLarge = 1 << 21;
 constexpr int kEarlyLM = 2048;
 constexpr int kEarlyLT = 2048;
 constexpr int kWarpLM = 128;  // one warp per polygon: up to 128 members and triangles
@@ -876,8 +879,9 @@ cudaError_t launch_long_early(const DevMesh& M, uint8_t* lab, int* tf, const int
                               const LongList& early, const LongList& Lg, int* loc, int* vstamp,
                               int epoch, int repair, int cap, Counters* C, cudaStream_t s,
                               bool pdl) {
-  const auto launch = M.m < kEarlyMesh ? launch_long_t<kEarlyThreads / 2, kEarlyLM, kEarlyLT>
-                                       : launch_long_t<kEarlyThreads, kEarlyLM, kEarlyLT>;
+  const auto launch = M.m < kEarlyMesh    ? launch_long_t<kEarlyThreads / 2, kEarlyLM, kEarlyLT>
+                      : M.m <= kEarlyLarge ? launch_long_t<kEarlyThreads, kEarlyLM, kEarlyLT>
+                                           : launch_long_t<kLongThreads, kLM, kLT>;
   return launch(M, lab, tf, seeds, P, F, pool, early, C->n_early, Lg, &C->n_long, loc, vstamp,
                 epoch, repair, cap, C, 2 * kEarlyMost, s, pdl);
 }

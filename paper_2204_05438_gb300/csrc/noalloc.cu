@@ -100,16 +100,16 @@ extern "C" polylla_status polylla_label_seeds_noalloc(const int64_t* d_xy, int64
   M.n = n_vertices;
   M.m = n_tri;
   // the error word, counters and look-back words start at zero
-  if (seed_tiles(n_tri) + 1 > kNoAllocTiles) return POLYLLA_ERR_INVALID_ARG;
+  if (seed_tiles(n_tri, false) + 1 > kNoAllocTiles) return POLYLLA_ERR_INVALID_ARG;
   cudaError_t e = cudaMemsetAsync(C, 0, sizeof(Counters), s);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)(seed_tiles(n_tri) + 1), s);
+    e = cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (size_t)(seed_tiles(n_tri, false) + 1), s);
   if (e == cudaSuccess) e = launch_label_max(M, d_lab, nullptr, C, grid_of(sms, (n_tri + 3) / 4, kBlock), s);
   if (e == cudaSuccess)
     e = launch_label_class(M, d_lab, nullptr, C, grid_of(sms, n_tri, kTriTile), s, true);
   if (e == cudaSuccess)
-    e = launch_seed_write(d_lab, n_tri, status, d_seeds, nullptr, M, nullptr, nullptr, C,
-                          grid_of(sms, n_tri, 16 * kTriTile), s, true);
+    e = launch_seed_write(d_lab, n_tri, status, d_seeds, nullptr, M, nullptr, nullptr, false, C, s,
+                          true);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_n_seeds, &C->n_seeds, sizeof(long long), cudaMemcpyDeviceToDevice, s);
   int err = 0;

@@ -25,6 +25,9 @@ constexpr long long kMaxTriangles = 1ll << 29;
 constexpr long long kMaxVertices = 1ll << 30;
 constexpr int kWalkThreads = 256;  // k_walk block
 constexpr int kEarlyMost = 256;    // seeds of either kind for blocks beside the walk, at most
+// Larger meshes leave all to the walk: the labels' extra work is then what hiding one region
+// saves (8M triangles of a mixture 441 us the run, 428 with blocks beside; 20M 872, 886).
+constexpr long long kBesideMost = 1ll << 23;
 constexpr unsigned kEarlyBit = 0x80000000u;  // of their entries
 constexpr int kLenChunk = 128;               // triangles per word of the length array
 constexpr int kWalkCap = 64;       // longer polygons go to one thread block each (long.cu)
@@ -260,14 +263,14 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
                                cudaStream_t s, bool pdl);
 // The ascending seed list (and each seed's terminal half-edge, if entry is
 // non-null), C->n_seeds and C->n_front in one pass:
-// look-back over `status` (seed_tiles(m) words, zero at the first use; left zero)
+// look-back over `status` (seed_tiles(m, small) words, for this and any smaller m;
+// zero at the first use, left zero)
 // with tickets from C->seed_ticket (zero at the start).
 // len, early (nullable): see k_seed_write.
 cudaError_t launch_seed_write(const uint8_t* lab, long long m, unsigned long long* status,
                               int* seeds, int* entry, const DevMesh& M, const unsigned* len,
-                              int* early, Counters* C, int grid, cudaStream_t s,
-                              bool pdl);
-long long seed_tiles(long long m);
+                              int* early, bool small, Counters* C, cudaStream_t s, bool pdl);
+long long seed_tiles(long long m, bool small);
 // Per polygon of the traversal (index = seed order), capacity m.
 struct PolyArrays {
   int* start;     // canonical start half-edge of the traversal polygon

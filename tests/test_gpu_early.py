@@ -53,6 +53,14 @@ def test_listed_seeds_about_the_limit(over):
     assert_parity(mesh)
 
 
+@pytest.mark.parametrize("m", [8191, 8192, 8193, 12288, 12289])
+def test_tiles_of_the_seed_pass(m):
+    """Sizes about whole tiles of 4096 triangles."""
+    mesh = strips(m - len(strips(1)["tri"]) + 1)
+    assert len(mesh["tri"]) == m
+    assert_parity(mesh)
+
+
 @pytest.mark.parametrize("k", [63, 64, 500, 2045, 2046, 2047, 2100])
 def test_long_regions_beside_the_walk(k):
     """Wheels of k triangles: about the walk's limit, and about what a block holds."""
