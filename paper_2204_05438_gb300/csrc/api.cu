@@ -275,8 +275,6 @@ polylla_status alloc_derived(polylla_mesh* h) {
   ALLOC(h->vtx_final, 3 * m);
   ALLOC(h->C, 1);
 #undef ALLOC
-  if (e == cudaSuccess)
-    e = cudaMallocHost(reinterpret_cast<void**>(&h->C_host), sizeof(Counters));
   // stamped arrays start empty (run stamps are never 0); look-back words start zero
   // (each pass leaves them zero).  The clears are waited for: the caller's first run
   // may be on any stream, and a clear that came late would take words from under it
@@ -343,10 +341,14 @@ long long derived_bytes(long long n, long long m) {
 // Waits for the handle's work and reads its counters.  The copy goes behind that work
 // into pinned memory and one wait covers both: a wait followed by a copy to pageable
 // memory cost a second round trip to the device (a run of 1,979 triangles and its
-// polygons: 102 us, now 89, with the binding's part).
+// polygons: 102 us, now 89, with the binding's part).  The pinned copy is made at the first
+// read: a server's slots never read, and pinning memory while other slots run held
+// them up (slots created in a served stream: its slowest request 29 ms).
 polylla_status read_counters(polylla_mesh* h, Counters* out) {
-  cudaError_t e = cudaMemcpyAsync(h->C_host, h->C, sizeof(Counters), cudaMemcpyDeviceToHost,
-                                  h->last_stream);
+  cudaError_t e = cudaSuccess;
+  if (!h->C_host) e = cudaMallocHost(reinterpret_cast<void**>(&h->C_host), sizeof(Counters));
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->C_host, h->C, sizeof(Counters), cudaMemcpyDeviceToHost, h->last_stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->last_stream);
   if (e != cudaSuccess) return cuda_status(e);
   *out = *h->C_host;
