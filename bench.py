@@ -47,16 +47,16 @@ FALLBACK_HBM_GBS = 6800.0
 # (source_hash(TRAFFIC_FILES)); reported as null once that code changes.
 TRAFFIC_FILES = ("final.cu", "label.cu", "long.cu", "polylla_internal.cuh", "trav.cu", "walk.cuh")
 NCU_TRAFFIC = {
-    "sources": "fe8214375f1b7185",
+    "sources": "df442eb742bdc2e3",
     # one ncu --set full capture per kernel on gmm16-5m (9,999,947 triangles),
     # scaled x2.0000 by triangle count to a gmm16-10m launch
-    "bytes": {"walk": int((311.370 + 70.850) * 1e6 * 19999948 / 9999947),
-              "out_write": int((90.156 + 27.965) * 1e6 * 19999948 / 9999947),
-              "label_class": int((130.077 + 80.119) * 1e6 * 19999948 / 9999947),
-              "label_max": int((200.068 + 8.866) * 1e6 * 19999948 / 9999947),
+    "bytes": {"walk": int((255.898 + 67.589) * 1e6 * 19999948 / 9999947),
+              "out_write": int((92.261 + 27.653) * 1e6 * 19999948 / 9999947),
+              "label_class": int((130.074 + 79.697) * 1e6 * 19999948 / 9999947),
+              "label_max": int((200.065 + 9.444) * 1e6 * 19999948 / 9999947),
               "seed_write": int((10.046 + 0.001) * 1e6 * 19999948 / 9999947),
-              "repair_one": int((83.686 + 3.596) * 1e6 * 19999948 / 9999947),
-              "repair_multi": int((15.205 + 0.003) * 1e6 * 19999948 / 9999947)},
+              "repair_one": int((83.471 + 3.305) * 1e6 * 19999948 / 9999947),
+              "repair_multi": int((22.755 + 0.002) * 1e6 * 19999948 / 9999947)},
 }
 
 
@@ -345,7 +345,7 @@ def run_ours(args, dist: Dist) -> dict | None:
     ls_ms = sum(kernels[k]["ms"] for k in label_seed)
     ls_bytes = sum(kernels[k]["alg_bytes"] for k in label_seed)
     ls_io = 24 * m + 16 * n + m + 4 * sizes["ns"]
-    # traversal: the successor pass and the walk together, against their own
+    # traversal: the walk, against its own
     # algorithmic bytes and against the survey's estimate of the traversal phase's
     # bytes (about 35 B per triangle: twin, label and origin reads over the visited
     # half-edges, the vertex and offset writes)

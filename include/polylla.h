@@ -111,7 +111,7 @@ typedef struct {
                              list holds, split by re-walking */
   int64_t n_one_chase;    /* one-tip polygons whose pieces could not be cut out of the
                              traversal's vertex sequence (a repeated vertex), split by
-                             chasing the successors */
+                             chasing the turns */
   int64_t n_multi_turn;   /* pieces of several-tip polygons whose smallest vertex
                              repeats, their half-edges found by turning */
   int64_t n_one_block;    /* polygons of a small mesh meshed, whole path, by one
@@ -368,7 +368,7 @@ polylla_status polylla_get_lepp(polylla_mesh_t mesh, const int32_t** d_region,
  * are captured into a CUDA graph on its first use (that call runs eagerly) and
  * replayed afterwards.  schedule: 0 .. polylla_batch_schedules()-1, or
  * POLYLLA_SCHEDULE_TUNED for the one polylla_batch_tune picked (tuning first if
- * needed).  A schedule sets the longest polygon walked by one thread (longer
+ * needed).  A schedule sets the longest polygon the walk places (longer
  * ones go to one thread block each) and how those blocks are sized (long_mode 0:
  * one large block per polygon; 1: small blocks first, several per SM, handing
  * the regions they cannot hold to large ones; 2: the same with one warp per
@@ -510,7 +510,7 @@ void polylla_debug_fail_alloc(int64_t k);
 /*
  * Test switch (Section 3.2.3's split, its rarer device paths): with enable != 0,
  * the reparation of this handle takes the paths normally kept for polygons with
- * a repeated vertex on every polygon -- one-tip pieces by chasing the successors
+ * a repeated vertex on every polygon -- one-tip pieces by chasing the turns
  * (counted in n_one_chase), several-tip pieces ordered by (origin, half-edge) with
  * half-edges found by turning (n_multi_turn), and each split's far node found
  * through turn(oj) -- so that tests can compare those paths with the oracle on any

@@ -9,7 +9,8 @@
 //           into the vertex pool, whose space is handed out per warp.  A polygon
 //           with tips is listed -- one tip (about 90% of them) or several -- so that
 //           the dependent loads of a split do not stall its warp; a longer one is
-//           left to one thread block (long.cu).
+//           left to one thread block (long.cu), and a seed listed by the seed pass,
+//           whose region may be long, to a block that runs beside the walk.
 //   k_repair_one    one thread per polygon with one tip: split it and cut the
 //           two pieces out of the vertex sequence the walk left in the pool.
 //   k_repair_multi  one warp per polygon with several tips: all split edges at once,
@@ -57,9 +58,11 @@ __device__ __forceinline__ long long warp_alloc(long long* counter, int need) {
 //   2. the passes backwards: each triangle's boundary edges, from its children's;
 //   3. the passes forwards: each triangle's place in its polygon, its children's, and
 //      its frontier edges into he[], polygon after polygon;
-//   4. the origins gathered, a lane per boundary edge; a lane per polygon scans them
-//      for the smallest (origin, half-edge) and the tips; then every lane stores its
-//      edges' origins, each polygon turned to start there, in one stretch of the pool.
+//   4. the origins gathered, a lane per boundary edge, and compared in shared memory:
+//      each polygon's smallest vertex and where it is (the half-edges only if it
+//      repeats), and the vertices that repeat two steps on, which tips do; then every
+//      lane stores its edges' origins, each polygon turned to start at its smallest,
+//      in one stretch of the pool.
 //
 // What bounds it: the latency of the queue's passes, ten on average for the 212
 // triangles of 32 regions, and the instructions issued (3,000 a warp and 32 seeds, 60
