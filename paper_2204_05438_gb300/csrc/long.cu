@@ -319,6 +319,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
   for (long long j = blockIdx.x; j < nl; j += gridDim.x) {
     const long long i = Lg.poly[early && j >= ne ? kEarlyMost + j - ne : j];
     const int t0 = seeds[i];
+    if (threadIdx.x == 0) {  // no output unless written below: the walk has not seen a listed seed
+      P.pcnt[i] = 0;
+      P.flen[i] = 0;
+    }
     if (t0 < 0 || t0 >= M.m) {  // (the same for the whole block)
       if (threadIdx.x == 0) set_error(C, POLYLLA_ERR_LIMIT, 115);
       continue;
@@ -452,8 +456,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_long(DevMesh M, uint8_t* lab, in
       P.start[i] = mem[c];
       P.len[i] = L;
       P.ntip[i] = nt;
-      P.pcnt[i] = 0;
-      P.flen[i] = 0;
       atomicAdd(reinterpret_cast<unsigned long long*>(&C->n_vtx_trav), (unsigned long long)L);
       if (early) count_early(L, nt, early, repair, M.m, 1ull, C);
       if (nt) {
