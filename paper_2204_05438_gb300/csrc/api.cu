@@ -73,7 +73,6 @@ struct polylla_mesh {
   long long* off_final = nullptr;
   int* vtx_final = nullptr;
   Counters* C = nullptr;
-  Counters* C_host = nullptr;  // pinned: where read_counters has them copied
 
   // the three kernels after the walk touch disjoint polygons: fork to two side
   // streams and join back (sequential in timing mode, for per-kernel times)
@@ -201,7 +200,6 @@ void free_all(polylla_mesh* h) {
     cudaEventDestroy(r.b);
   }
   for (auto e : h->event_pool) cudaEventDestroy(e);
-  if (h->C_host) cudaFreeHost(h->C_host);
   for (int k = 0; k < 2; ++k) {
     if (h->side[k]) cudaStreamDestroy(h->side[k]);
     if (h->join[k]) cudaEventDestroy(h->join[k]);
@@ -338,20 +336,17 @@ long long derived_bytes(long long n, long long m) {
   return bytes;
 }
 
-// Waits for the handle's work and reads its counters.  The copy goes behind that work
-// into pinned memory and one wait covers both: a wait followed by a copy to pageable
-// memory cost a second round trip to the device (a run of 1,979 triangles and its
-// polygons: 102 us, now 89, with the binding's part).  The pinned copy is made at the first
-// read: a server's slots never read, and pinning memory while other slots run held
-// them up (slots created in a served stream: its slowest request 29 ms).
+// Waits for the handle's work and reads its counters, into the caller's own copy: a copy
+// to pageable memory, queued behind that work, returns when it has arrived, so one wait
+// covers both.  A wait and then a copy made a second round trip to the device (1,979
+// triangles, the run and its polygons: 103 us, 98 with one).  A pinned copy kept with the
+// handle was no faster, took 8 to 120 us to make, and would be shared by two threads that
+// read one handle.
 polylla_status read_counters(polylla_mesh* h, Counters* out) {
-  cudaError_t e = cudaSuccess;
-  if (!h->C_host) e = cudaMallocHost(reinterpret_cast<void**>(&h->C_host), sizeof(Counters));
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->C_host, h->C, sizeof(Counters), cudaMemcpyDeviceToHost, h->last_stream);
+  cudaError_t e =
+      cudaMemcpyAsync(out, h->C, sizeof(Counters), cudaMemcpyDeviceToHost, h->last_stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->last_stream);
   if (e != cudaSuccess) return cuda_status(e);
-  *out = *h->C_host;
   if (out->error) return (polylla_status)out->error;
   return POLYLLA_OK;
 }
