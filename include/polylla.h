@@ -112,8 +112,9 @@ typedef struct {
   int64_t n_one_chase;    /* one-tip polygons whose pieces could not be cut out of the
                              traversal's vertex sequence (a repeated vertex), split by
                              chasing the turns */
-  int64_t n_multi_turn;   /* pieces of several-tip polygons whose smallest vertex
-                             repeats, their half-edges found by turning */
+  int64_t n_multi_turn;   /* pieces, of polygons split by the several-tip kernel, whose
+                             smallest vertex repeats: the smallest half-edge there is
+                             their start */
   int64_t n_one_block;    /* polygons of a small mesh meshed, whole path, by one
                              thread block (polylla_run; see polylla_set_one_block) */
 } polylla_stats;
@@ -511,9 +512,8 @@ void polylla_debug_fail_alloc(int64_t k);
  * Test switch (Section 3.2.3's split, its rarer device paths): with enable != 0,
  * the reparation of this handle takes the paths normally kept for polygons with
  * a repeated vertex on every polygon -- one-tip pieces by chasing the turns
- * (counted in n_one_chase), several-tip pieces ordered by (origin, half-edge) with
- * half-edges found by turning (n_multi_turn), and each split's far node found
- * through turn(oj) -- so that tests can compare those paths with the oracle on any
+ * (counted in n_one_chase), several-tip pieces with every successor found by
+ * turning (each piece counted in n_multi_turn) -- so that tests can compare those paths with the oracle on any
  * mesh.  The polygons are the same either way.  While it is on, polylla_run
  * takes the multi-kernel path at every mesh size.  Errors:
  * POLYLLA_ERR_INVALID_ARG for a null handle.

@@ -56,7 +56,7 @@ struct Counters {
   long long n_long_seq;   // long regions too large for a block, walked by one thread
   long long n_multi_seq;  // several-tip polygons with more tips than the node list holds
   long long n_one_chase;  // one-tip polygons split by chasing (a repeated vertex)
-  long long n_multi_turn; // several-tip pieces with a repeated smallest vertex
+  long long n_multi_turn; // pieces of k_repair_multi with a repeated smallest vertex
   long long seed_ticket;  // tile tickets of the seed compaction's look-back
   long long seed_done;    // its completed look-backs (the last one clears the status)
   long long out_done;     // the output pass's completed look-backs (likewise)

@@ -770,11 +770,12 @@ struct SplitBuf {
 };
 
 // Returns the number of pieces (their records in F from *foff), or -1; every lane of
-// the warp calls it.  hs: the polygon's L half-edges, overwritten with the pieces.
+// the warp calls it.  *by_half_edge grows by the pieces whose smallest vertex repeats (all,
+// if rare).  hs: the polygon's L half-edges, overwritten with the pieces.
 __device__ __forceinline__ int split_by_warp(const DevMesh& M, uint8_t* lab, int* tf, SplitBuf& B,
                                              int L, int nt, int* hs, long long off,
                                              const FinalPieces& F, int rare, Counters* C,
-                                             long long* foff) {
+                                             long long* foff, unsigned* by_half_edge) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
@@ -881,10 +882,12 @@ __device__ __forceinline__ int split_by_warp(const DevMesh& M, uint8_t* lab, int
   // a lane per side of each split edge walks its piece
   const bool side = lane < 2 * ns;
   int name = 255, len = 0, least = 0x7fffffff, start = 0;
+  bool again = false;  // the smallest vertex repeats
   if (side) {
     int a = L + lane;
     do {
       const int o = B.v[a];
+      again = o == least || (again && o > least);
       if (o < least || (o == least && B.h[a] < B.h[start])) {
         least = o;
         start = a;
@@ -898,6 +901,7 @@ __device__ __forceinline__ int split_by_warp(const DevMesh& M, uint8_t* lab, int
   const unsigned owners = __ballot_sync(full, side && name == L + lane);
   const int np = __popc(owners);
   if (np != ns + 1) return -1;
+  *by_half_edge += __popc(owners & __ballot_sync(full, again || rare));
   // the piece of each side, numbered by name; each piece's start and length
   const int piece = side ? __popc(owners & ((1u << (name - L)) - 1u)) : 0;
   if (owners >> lane & 1u) {
@@ -970,8 +974,8 @@ __global__ void __launch_bounds__(kRsThreads) k_repair_multi(DevMesh M, uint8_t*
     if (nt >= 2 && nt <= kRsMaxSplit && L >= 3 && L <= kWalkCap && P.pbase[i] == 1) {
       const long long off = P.pos[i];
       if (off >= 0 && off + L + 2 * nt <= pool.cap)
-        cnt = split_by_warp(M, lab, tf, s_buf[warp], L, nt, pool.v + off, off, F, rare, C, &foff);
-      if (rare && cnt > 0) st_turn += cnt;
+        cnt = split_by_warp(M, lab, tf, s_buf[warp], L, nt, pool.v + off, off, F, rare, C, &foff,
+                            &st_turn);
     } else if (nt > kRsMaxSplit && L >= 3) {
       if (lane == 0) {  // more tips than the nodes hold: one thread, piece by piece
         ++st_seq;
