@@ -64,7 +64,8 @@ struct polylla_mesh {
   FinalPieces F{};
   Pool pool{};
   LongList Dm{};          // polygons with several tips
-  LongList Lg2{};         // long polygons the small blocks hand to the large ones
+  LongList Lg2{};         // long polygons the small blocks hand to the large ones, or (long_mode
+                          // 0) the seeds listed for blocks beside the walk
   int epoch = 0;
   unsigned long long* seed_status = nullptr;  // look-back words of the seed pass
   unsigned long long* out_status = nullptr;   // look-back words of the output pass
@@ -360,9 +361,12 @@ polylla_status check_handle(polylla_mesh* h) {
 }
 
 // ---------------------------------------------------------------- phases
-// Whether blocks beside the walk take the regions that may be long.
+// Whether blocks beside the walk take the regions that may be long.  Their list stands in
+// Lg2.poly from the seeds to the last pass over the polygons, so not in a long_mode that
+// hands regions on through Lg2 (a batch's schedules).
 bool beside(const polylla_mesh* h) {
-  return h->beside && !h->rare_paths && h->M.m >= 2 * kEarlyMost && h->M.m <= kBesideMost;
+  return h->beside && h->long_mode == 0 && !h->rare_paths && h->M.m >= 2 * kEarlyMost &&
+         h->M.m <= kBesideMost;
 }
 
 polylla_status do_label(polylla_mesh* h, cudaStream_t s) {
