@@ -123,8 +123,6 @@ def algorithmic_bytes(name: str, s: dict) -> float:
         # record (count, length, pos) out, per vertex its origin in and pool out, and
         # start, length, tips and tip for each polygon with tips
         "walk": 12 * m + 4 * ns + 8 * nv0 + 16 * ns + 16 * s.get("ntp", 0),
-        # per polygon its piece count and length
-        "out_tiles": 8 * ns,
         # per polygon record in, pool in, offsets and vertices out
         "out_write": 16 * ns + 8 * nv + 8 * (npoly + 1),
     }.get(name, 0.0)

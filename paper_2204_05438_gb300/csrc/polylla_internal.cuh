@@ -1,5 +1,5 @@
 // Internal declarations of the GB300 mesher library: device-side data, half-edge
-// helpers, block-level scans and the launchers of every kernel.
+// helpers, the look-back scan and the launchers of every kernel.
 //
 // Mesh layout (Section 2 of the paper, with an explicit half-edge twin): half-edge
 // h = 3t+k of triangle t runs from tri[h] to tri[3t+(k+1)%3]; twin[h] is the
@@ -82,7 +82,6 @@ struct DevMesh {
 };
 
 // ----------------------------------------------------------------- half-edges
-__device__ __forceinline__ int he_tri(int h) { return h / 3; }
 __device__ __forceinline__ int he_next(int h) {
   const int t3 = 3 * (h / 3);
   return (h - t3 == 2) ? t3 : h + 1;
@@ -91,46 +90,8 @@ __device__ __forceinline__ int he_prev(int h) {
   const int t3 = 3 * (h / 3);
   return (h == t3) ? t3 + 2 : h - 1;
 }
-// Frontier flag of half-edge h read from the label byte of its triangle.  Plain
-// loads: reparation updates label bytes inside the same kernel.
-__device__ __forceinline__ bool lab_frontier(const uint8_t* lab, int h) {
-  const int t = h / 3;
-  return (lab[t] >> (2 + (h - 3 * t))) & 1;
-}
-
 __device__ __forceinline__ void set_error(Counters* c, int code, int info) {
   if (atomicCAS(&c->error, 0, code) == 0) c->err_info = info;
-}
-
-// ----------------------------------------------------------------- block scans
-// Exclusive scan over the kBlock threads of a block; returns the thread's prefix
-// and writes the block total.  `sh` needs kBlock/32 entries.  Contains barriers:
-// every thread of the block must call it.
-template <typename T>
-__device__ __forceinline__ T block_exclusive_scan(T v, T* total, T* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T x = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    T y = __shfl_up_sync(0xffffffffu, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) sh[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    T w = (lane < kBlock / 32) ? sh[lane] : T(0);
-#pragma unroll
-    for (int d = 1; d < kBlock / 32; d <<= 1) {
-      T y = __shfl_up_sync(0xffffffffu, w, d);
-      if (lane >= d) w += y;
-    }
-    if (lane < kBlock / 32) sh[lane] = w;
-  }
-  __syncthreads();
-  const T before = warp ? sh[warp - 1] : T(0);
-  *total = sh[kBlock / 32 - 1];
-  __syncthreads();
-  return before + x - v;
 }
 
 // ------------------------------------------------------------ look-back scan

@@ -21,9 +21,6 @@
 
 namespace polylla {
 
-constexpr int kTipFlag = 1 << 31;
-constexpr int kSuccMask = 0x7fffffff;
-
 __device__ __forceinline__ int tf_twin(int x) { return x & 0x7fffffff; }
 
 // Canonical key of a frontier half-edge: (origin vertex, half-edge id).
