@@ -229,12 +229,12 @@ __global__ void __launch_bounds__(kBlock, 5) k_label_class(DevMesh M, uint8_t* l
         unsigned nbm = 0;  // bit k: edge k is also the longest edge of the neighbour
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
+          if (tw[3 * j + k] >= H) {  // a border edge from here on: every tf word is frontier or a twin
+            set_error(C, POLYLLA_ERR_RANGE, 11);
+            tw[3 * j + k] = -1;
+          }
           const int gk = tw[3 * j + k];
           if (gk >= 0) {
-            if (gk >= H) {
-              set_error(C, POLYLLA_ERR_RANGE, 11);
-              continue;
-            }
             const int gt = gk / 3;
             const int nb = lab[gt] & 3;
             nbm |= (unsigned)(nb == gk - 3 * gt) << k;

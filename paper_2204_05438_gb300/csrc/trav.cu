@@ -165,7 +165,10 @@ __global__ void __launch_bounds__(kWalkThreads, 4) k_walk(DevMesh M, const int* 
     // A listed seed of a kind the blocks have is theirs.  The kind comes from the twin array,
     // which nothing writes: the blocks mark split edges in tf at the same time, and one may be
     // a listed region's own terminal edge, whose word then looks like a border's.
-    if (raw < 0 && e0 >= 0 && (__ldg(M.twin + e0) < 0 ? early0 : early1)) e0 = -1;
+    if (raw < 0 && e0 >= 0) {
+      const int g = __ldg(M.twin + e0);  // (out of range: a border's, to the label pass)
+      if (g < 0 || g >= H ? early0 : early1) e0 = -1;
+    }
     int x0 = e0 >= 0 ? __ldg(tf + e0) : -1;  // (of regions that only the walk has)
     bool big = false;  // too long for a walk: left to a thread block
     for (int b0 = 0; b0 < per && base + b0 < n;) {

@@ -50,3 +50,26 @@ def test_no_polygon_of_a_region_with_an_error():
     np.testing.assert_array_equal(got[:before + 1], ref["off"][:before + 1])
     np.testing.assert_array_equal(np.diff(got[before:before + 3]), [0, 3])
     M.close()
+
+
+@pytest.mark.parametrize("edge", ["longest", "other"])
+def test_twin_out_of_range_is_a_border_to_every_kernel(edge):
+    """A twin one past the last half-edge, not validated: the label pass reports it and
+    marks the edge frontier, so that no later kernel follows it."""
+    mesh = meshgen.generate("uniform", 3000, 1 << 18, 46)
+    ref = oracle.full(mesh)
+    m = len(mesh["tri"])
+    twin = np.asarray(mesh["twin"]).reshape(-1, 3)
+    t = int(np.nonzero((twin >= 0).all(axis=1))[0][5])  # an interior triangle
+    k = (int(ref["label"]["max_edge"][t]) + (edge == "other")) % 3
+    M = pg.from_numpy(mesh)
+    M.set_one_block(0)
+    M.twin.view(-1)[3 * t + k] = 3 * m
+    torch.cuda.synchronize()
+    M.label()
+    assert int(M.labels()[t]) >> (2 + k) & 1
+    M.seeds(), M.traverse(), M.repair()
+    with pytest.raises(pg.PolyllaError) as e:
+        M.polygons()
+    assert e.value.code == 2  # POLYLLA_ERR_RANGE
+    M.close()
