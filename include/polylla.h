@@ -96,19 +96,21 @@ typedef struct {
   int64_t n_poly;         /* polygons after reparation */
   int64_t n_vtx;          /* their total length */
   /* Which device path handled the polygons of the last traversal / reparation
-   * pass (every path gives the same polygons; these show which ones ran; a polygon
-   * that a block took beside the walk counts as what the walk would have made it): */
-  int64_t n_long;         /* polygons longer than the thread walk's cap (and, on
-                             meshes of fewer than 2^16 triangles, polygons with three
-                             or more tips), walked and split by one thread block each */
+   * pass (every path gives the same polygons; these show which ones ran; in n_long,
+   * n_one_tip, n_multi_tip and n_multi_seq a polygon that a block took beside the walk
+   * counts as what the walk would have made it): */
+  int64_t n_long;         /* polygons longer than the walk's cap (and, on meshes of fewer
+                             than 2^16 triangles, polygons with nine or more tips; and
+                             those of a warp whose polygons have more tips in all than
+                             its list holds), walked and split by one thread block each */
   int64_t n_long_handoff; /* of those, regions a small block could not hold and
                              handed to a large one (batch schedules with long_mode 1, 2) */
   int64_t n_long_seq;     /* of those, regions too large for any block's shared
                              memory, walked and split by one thread */
   int64_t n_one_tip;      /* polygons with exactly one tip, split by the one-tip kernel */
-  int64_t n_multi_tip;    /* polygons with several tips, split in shared memory */
-  int64_t n_multi_seq;    /* of those, polygons with more tips than the shared node
-                             list holds, split by re-walking */
+  int64_t n_multi_tip;    /* polygons with several tips, split by one warp each */
+  int64_t n_multi_seq;    /* of those, polygons with more tips than a warp splits
+                             together (eight), split by one thread, piece by piece */
   int64_t n_one_chase;    /* one-tip polygons whose pieces could not be cut out of the
                              traversal's vertex sequence (a repeated vertex), split by
                              chasing the turns */
@@ -417,9 +419,10 @@ polylla_status polylla_batch_destroy(polylla_batch_t batch);
  * Capacity handles and asynchronous results (for callers that reuse device
  * state across meshes, such as the server below).
  *
- * polylla_mesh_footprint: device bytes a handle for n vertices and m triangles
- * allocates (owns_inputs != 0: also its input arrays, as polylla_mesh_create_host
- * does); -1 for invalid sizes.  No device call.
+ * polylla_mesh_footprint: device bytes to reserve for a handle for n vertices and m
+ * triangles, at least what it allocates (owns_inputs != 0: also its input arrays, as
+ * polylla_mesh_create_host does, and 8n + 24m + 4 bytes for the twin construction, whose
+ * table takes 16m + 32 at most); -1 for invalid sizes.  No device call.
  * polylla_mesh_set_size: for a handle created by polylla_mesh_create_host, the
  * size of the next mesh (at most its creation sizes); the phases restart.
  * polylla_mesh_inputs: the device input arrays of such a handle, to fill
@@ -513,8 +516,8 @@ void polylla_debug_fail_alloc(int64_t k);
  * the reparation of this handle takes the paths normally kept for polygons with
  * a repeated vertex on every polygon -- one-tip pieces by chasing the turns
  * (counted in n_one_chase), several-tip pieces with every successor found by
- * turning (each piece counted in n_multi_turn) -- so that tests can compare those paths with the oracle on any
- * mesh.  The polygons are the same either way.  While it is on, polylla_run
+ * turning (each piece counted in n_multi_turn) -- so that tests can compare those
+ * paths with the oracle on any mesh.  The polygons are the same either way.  While it is on, polylla_run
  * takes the multi-kernel path at every mesh size.  Errors:
  * POLYLLA_ERR_INVALID_ARG for a null handle.
  */

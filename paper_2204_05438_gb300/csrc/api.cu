@@ -516,7 +516,8 @@ polylla_status do_repair(polylla_mesh* h, cudaStream_t s) {
 // Scratch of the twin construction, for handles that may build their twin.
 polylla_status alloc_twin_scratch(polylla_mesh* h) {
   const long long m = h->M.m, n = h->M.n;
-  // far more vertices than triangles (four and more each) are refused
+  // far more vertices than triangles (four and more each) are refused, as they have been: the
+  // table itself would do for them
   if ((n + kTriTile - 1) / kTriTile > (m + kPolyTile - 1) / kPolyTile)
     return POLYLLA_ERR_INVALID_ARG;
   return cuda_status(dalloc(&h->tw_table, twin_words(m)));

@@ -293,11 +293,14 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // With `early`, the seeds whose regions may be long are listed (their entries carry
 // kEarlyBit): those whose terminal edge is a border edge (the label's frontier bit of
 // the longest edge; the slivers along a hull), and those whose terminal edge is at least a
-// 16th of the mesh's longest edge (the gaps between clusters).  On uniform and mixture
-// meshes of 1,000 to 1M points, 17-38 seeds of the first kind and 40-60 of the second
-// include every region of more than kWalkCap boundary edges.  A kind with more than
-// kEarlyMost seeds (a domain with holes; a mesh of edges all alike) says nothing, and
-// its seeds are the walk's like all others.
+// 16th of the mesh's longest edge (the gaps between clusters).  Counted on the host on
+// uniform and mixture meshes of 1,000 to 1M points: 13-42 seeds of the first kind, and of
+// the second 15-45 on mixtures, 184-237 on 1,000 uniform points, 28 or fewer on 5,000 and
+// none from 20,000 on; every region of more than kWalkCap boundary edges is among them.  A
+// kind with more than kEarlyMost seeds says nothing, and its seeds are the walk's like all
+// others: a mesh of edges all alike, or the border kind of a domain with holes (183-194
+// seeds at 20,000 uniform points, 295 at 60,000, 339 at 100,000), whose long regions are
+// then walked after the others as on larger meshes.
 constexpr int kSeedPer = 16;
 constexpr int kSeedSpan = kBlock * kSeedPer;   // triangles per sub-tile
 // Sub-tiles per look-back tile: 4, or 1 on meshes of at most kSeedSmall triangles, where

@@ -54,7 +54,7 @@ struct Counters {
   long long n_multi_early; // with several
   long long n_long2;      // long polygons handed from the small blocks to the large ones
   long long n_long_seq;   // long regions too large for a block, walked by one thread
-  long long n_multi_seq;  // several-tip polygons with more tips than the node list holds
+  long long n_multi_seq;  // several-tip polygons with more tips than a warp splits together
   long long n_one_chase;  // one-tip polygons split by chasing (a repeated vertex)
   long long n_multi_turn; // pieces of k_repair_multi with a repeated smallest vertex
   long long seed_ticket;  // tile tickets of the seed compaction's look-back
@@ -269,11 +269,12 @@ struct LongList {
   long long cap;
 };
 
-// One thread per seed: walk (<= kWalkCap) and, if `repair`, list polygons with
+// A warp per 32 seeds: their polygons (<= kWalkCap) and, if `repair`, lists of those with
 // tips.  cap: polygons longer than cap (16, 32, 48 or 64) go to the long-polygon
 // blocks; with tips_to_long > 0 (small meshes), so do polygons with that many tips
-// or more when `repair` (the block splits their tips in parallel; one thread would
-// split them one after another).
+// or more when `repair` (more than kRsMaxSplit: a block splits their tips in parallel, one
+// thread would split them one after another), and so do the polygons of a warp with more
+// tips than its list holds.  beside: blocks beside the walk have the listed seeds.
 constexpr int kRsMaxSplit = 8;  // tips that a warp splits together (k_repair_multi)
 constexpr long long kSmallMeshTri = 1ll << 16;  // meshes below this: more go to blocks
 cudaError_t launch_walk(const DevMesh& M, const int* tf, const int* entry, const PolyArrays& P,

@@ -41,6 +41,9 @@ constexpr unsigned kTwinRandom = 64;          // words tried anywhere
 constexpr unsigned kTwinFree = 0xffffffffu;
 constexpr unsigned kTwinClosed = 0x80000000u;
 
+// (the multipliers here and in tile_slot: a prime next to 2^32 over the golden ratio, and the
+// low word of 2^64 over it; the two of MurmurHash3's 32-bit finaliser, A. Appleby, public
+// domain; 0x7feb352d from C. Wellons' search for 32-bit mixers, public domain)
 __device__ __forceinline__ unsigned twin_hash(unsigned a, unsigned b, unsigned i) {
   unsigned x = a * 0x9e3779b1u ^ (b + i * 0x7f4a7c15u) * 0x85ebca6bu;
   x ^= x >> 15;
