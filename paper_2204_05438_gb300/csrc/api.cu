@@ -337,17 +337,20 @@ long long derived_bytes(long long n, long long m) {
   return bytes;
 }
 
-// Waits for the handle's work and reads its counters, into the caller's own copy: a copy
-// to pageable memory, queued behind that work, returns when it has arrived, so one wait
-// covers both.  A wait and then a copy made a second round trip to the device (1,979
-// triangles, the run and its polygons: 103 us, 98 with one).  A pinned copy kept with the
-// handle was no faster, took 8 to 120 us to make, and would be shared by two threads that
-// read one handle.
+// Waits for the handle's work and reads its counters, into the caller's own copy: the copy
+// is queued behind that work and one wait covers both.  A wait and then a copy made a second
+// round trip to the device (1,979 triangles, the run and its polygons: 103 us against 98).  A
+// pinned copy kept with the handle, in place of the pageable one, saves a further 1 us a
+// read (53.9 us for the polygons' read, 55.0), but takes 8 to 120 us to make and up to 170 to
+// free, and two threads that read one handle would share it.
 polylla_status read_counters(polylla_mesh* h, Counters* out) {
   cudaError_t e =
       cudaMemcpyAsync(out, h->C, sizeof(Counters), cudaMemcpyDeviceToHost, h->last_stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->last_stream);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // a refused read (a stream under capture) is not the next launch's error
+    return cuda_status(e);
+  }
   if (out->error) return (polylla_status)out->error;
   return POLYLLA_OK;
 }

@@ -298,7 +298,7 @@ cudaError_t launch_label_class(const DevMesh& M, uint8_t* lab, int* tf, Counters
 // the second 15-45 on mixtures, 184-237 on 1,000 uniform points, 28 or fewer on 5,000 and
 // none from 20,000 on; every region of more than kWalkCap boundary edges is among them.  A
 // kind with more than kEarlyMost seeds says nothing, and its seeds are the walk's like all
-// others: a mesh of edges all alike, or the border kind of a domain with holes (183-194
+// others: a mesh of edges all alike, or the border kind of a domain with holes (120-218
 // seeds at 20,000 uniform points, 295 at 60,000, 339 at 100,000), whose long regions are
 // then walked after the others as on larger meshes.
 constexpr int kSeedPer = 16;

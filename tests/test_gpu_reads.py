@@ -1,6 +1,8 @@
-"""Reading a handle's results: by several threads at once, with nothing allocated."""
+"""Reading a handle's results: by several threads at once, with nothing allocated, and not
+under a stream capture."""
 from __future__ import annotations
 
+import ctypes
 import threading
 
 import numpy as np
@@ -66,4 +68,30 @@ def test_phases_and_reads_allocate_nothing():
         assert e.value.code == OOM
     finally:
         pg.debug_fail_alloc(0)
+    M.close()
+
+
+@pytest.mark.parametrize("mode", [0, 2], ids=["global", "relaxed"])
+def test_read_under_capture_is_refused(mode):
+    """A read waits for the device, which a stream capture does not allow: it fails, and it
+    leaves no graph behind that would write to the read's memory."""
+    rt = ctypes.CDLL(f"libcudart.so.{torch.version.cuda.split('.')[0]}")
+    mesh = meshgen.generate("uniform", 5_000, 1 << 20, 93)
+    ref = oracle.run(mesh)
+    M = pg.from_numpy(mesh)
+    s = torch.cuda.Stream()
+    M.run(s)
+    M.polygons()
+    at, graph = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(at, mode) == 0
+    M.run(s)
+    with pytest.raises(pg.PolyllaError):
+        M.polygons()
+    assert rt.cudaStreamEndCapture(at, ctypes.byref(graph)) != 0
+    assert not graph.value
+    rt.cudaGetLastError()
+    M.run(s)
+    off, vtx = (t.cpu().numpy() for t in M.polygons())
+    np.testing.assert_array_equal(off, ref["off"])
+    np.testing.assert_array_equal(vtx, ref["vtx"])
     M.close()
