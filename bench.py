@@ -47,16 +47,16 @@ FALLBACK_HBM_GBS = 6800.0
 # (source_hash(TRAFFIC_FILES)); reported as null once that code changes.
 TRAFFIC_FILES = ("final.cu", "label.cu", "long.cu", "polylla_internal.cuh", "trav.cu", "walk.cuh")
 NCU_TRAFFIC = {
-    "sources": "df442eb742bdc2e3",
+    "sources": "138183950b78dbcc",
     # one ncu --set full capture per kernel on gmm16-5m (9,999,947 triangles),
     # scaled x2.0000 by triangle count to a gmm16-10m launch
-    "bytes": {"walk": int((255.898 + 67.589) * 1e6 * 19999948 / 9999947),
-              "out_write": int((92.261 + 27.653) * 1e6 * 19999948 / 9999947),
-              "label_class": int((130.074 + 79.697) * 1e6 * 19999948 / 9999947),
-              "label_max": int((200.065 + 9.444) * 1e6 * 19999948 / 9999947),
-              "seed_write": int((10.046 + 0.001) * 1e6 * 19999948 / 9999947),
-              "repair_one": int((83.471 + 3.305) * 1e6 * 19999948 / 9999947),
-              "repair_multi": int((22.755 + 0.002) * 1e6 * 19999948 / 9999947)},
+    "bytes": {"walk": int((255.927 + 67.367) * 1e6 * 19999948 / 9999947),
+              "out_write": int((92.462 + 27.438) * 1e6 * 19999948 / 9999947),
+              "label_class": int((130.076 + 80.143) * 1e6 * 19999948 / 9999947),
+              "label_max": int((200.068 + 9.264) * 1e6 * 19999948 / 9999947),
+              "seed_write": int((10.046 + 0.000) * 1e6 * 19999948 / 9999947),
+              "repair_one": int((83.467 + 3.239) * 1e6 * 19999948 / 9999947),
+              "repair_multi": int((22.743 + 0.003) * 1e6 * 19999948 / 9999947)},
 }
 
 
